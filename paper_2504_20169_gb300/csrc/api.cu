@@ -161,6 +161,33 @@ void mean_equilibrium(const double* w, double r, const lbm_bc_params& bp, double
 
 int halo_of(int q) { return q == 9 ? 1 : 3; }
 
+// Fixed-point constants of an FP64 context (fixed.cuh). They stay off where that arithmetic does
+// not apply: omega outside (0, 2), or a mean state outside its range.
+template <class S>
+void fixed_consts(const double* w, double r, double omega, const lbm_bc_params& bp,
+                  const double* fbar, fx::Consts& c) {
+  std::memset(&c, 0, sizeof c);
+  auto units = [](long double v, int e) { return (fx::i64)std::llrint(std::ldexp(v, e)); };
+  c.r2 = r * r;
+  c.inv_r2 = 1.0 / c.r2;
+  if (!(omega > 0.0) || !(omega < 2.0)) return;
+  const double lg = std::log2(bp.rho0);
+  if (!(std::fabs(lg) < 60.0)) return;
+  c.E = (int)std::lround(lg);
+  c.om = fx::split(units(omega, 61));
+  for (int s = 0; s < S::NSHELL; ++s) {
+    const long double v = std::ldexp((long double)w[S::shell_first(s)], fx::shell_k<S>(s));
+    if (!(v > 0.5L && v < 1.0L)) return;
+    c.w[s] = fx::split(units(v, 62));
+    for (int i = S::shell_first(s); i < S::shell_first(s) + S::shell_size(s); ++i) {
+      const long double f = std::ldexp((long double)fbar[i], fx::shell_fe<S>(s) - c.E);
+      if (!(std::fabs(f) < std::ldexp(1.0L, 60))) return;
+      c.eqbar[i] = (fx::i64)std::llrint(f);
+    }
+  }
+  c.on = 1;
+}
+
 }  // namespace
 
 void lbm::set_global_error(const std::string& msg) { g_create_error = msg; }
@@ -553,6 +580,9 @@ lbm_status lbm_create(const lbm_grid* grid, lbm_stencil stencil, double tau, int
   }
   d.cd.r = ctx->r; d.cd.r2 = ctx->r * ctx->r; d.cd.omega = ctx->omega;
   d.cd.sigma_max = sg.sigma_max; d.cd.power = sg.power; d.cd.split = sg.split;
+  if (q == 37) fixed_consts<D2Q37>(ctx->w, ctx->r, ctx->omega, bp, fbar, d.cd.fx);
+  else if (q == 17) fixed_consts<D2Q17>(ctx->w, ctx->r, ctx->omega, bp, fbar, d.cd.fx);
+  else fixed_consts<D2Q9>(ctx->w, ctx->r, ctx->omega, bp, fbar, d.cd.fx);
   d.cf.r = (float)ctx->r; d.cf.r2 = (float)(ctx->r * ctx->r); d.cf.omega = (float)ctx->omega;
   d.cf.sigma_max = (float)sg.sigma_max; d.cf.power = sg.power; d.cf.split = sg.split;
   if (ctx->ops.prepare(ctx->w) != cudaSuccess) return oom("kernel attributes");

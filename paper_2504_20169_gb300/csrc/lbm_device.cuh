@@ -24,6 +24,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "fixed.cuh"
 #include "stencils.cuh"
 
 namespace lbm {
@@ -57,7 +58,13 @@ __host__ __device__ inline bool has_pml(const Geom& g) { return (g.Ww | g.We | g
 // Lattice and physics constants in the arithmetic type of a kernel. eqbar holds the
 // equilibrium of the PML mean state (Eq. decomp-NJ) in the storage representation.
 template <class Real>
-struct Consts {
+struct FixedConsts {};
+template <>
+struct FixedConsts<double> {
+  fx::Consts fx;     // the fixed-point form of an FP64 context's constants
+};
+template <class Real>
+struct Consts : FixedConsts<Real> {
   Real w[kMaxQ];
   Real eqbar[kMaxQ];
   Real r, r2, omega, sigma_max;
@@ -364,9 +371,79 @@ __device__ inline void load_pop(Real (&p)[S::Q], const Real* __restrict__ A, con
   }
 }
 
+// Populations of an FP64 node as fixed-point integers; false if one is out of their range.
+template <class S, bool STREAM>
+__device__ __forceinline__ bool load_fixed(fx::i64 (&F)[S::Q], const double* __restrict__ A,
+                                           const Geom& g, const fx::Consts& c, long long idx) {
+  int low = 1 << 20;
+  fx::unroll<S::NSHELL>([&](auto s) {
+    fx::unroll<S::shell_size(s)>([&](auto h) {
+      constexpr int i = S::shell_first(s) + h;
+      const long long src = STREAM ? pull_src(g, idx, S::ex(i), S::ey(i)) : idx;
+      F[i] = fx::load(__ldg(A + (long long)i * g.plane + src), fx::shell_fe<S>(s), c.E, low);
+    });
+  });
+  return low >= 3;
+}
+
+// put(i, s, feq) for every direction i (of shell s; both integral constants) with its
+// equilibrium in fixed point.
+template <class S, class Put>
+__device__ __forceinline__ void each_equilibrium(const fx::Consts& c, const fx::Site& k,
+                                                 fx::i64 rho58, Put put) {
+  fx::unroll<S::NSHELL>([&](auto s) {
+    constexpr int i0 = S::shell_first(s), n = S::shell_size(s);
+    const fx::Limbs wr = fx::shell_weight<S>(c, s, rho58);
+    if constexpr (n == 1) {
+      put(std::integral_constant<int, i0>(), s, fx::equilibrium(k.A0, wr));
+    } else {
+      const fx::Shell sh = fx::shell<S>(fx::shell_far<S>(s) ? fx::coarse<S::ORDER>(k) : k, s);
+      fx::unroll<n / 2>([&](auto h) {
+        constexpr int ip = i0 + h, im = ip + n / 2;
+        fx::i64 even, odd;
+        fx::factor<S>(sh, s, S::ex(ip), S::ey(ip), even, odd);
+        put(std::integral_constant<int, ip>(), s, fx::equilibrium(even + odd, wr));
+        put(std::integral_constant<int, im>(), s, fx::equilibrium(even - odd, wr));
+      });
+    }
+  });
+}
+
+// The macroscopic state of a fixed-point node in the form that the FP64 code keeps.
+__device__ __forceinline__ Macro<double> macro_of(const fx::State& u, const fx::Consts& c) {
+  Macro<double> m;
+  m.rho = double(u.rho) * fx::double_of((fx::u64)(1023 - 58 + c.E) << 52);
+  m.drho = m.rho - 1.0;
+  m.inv_rho = 0.0;   // not used by the callers
+  m.urx = u.X;
+  m.ury = u.Y;
+  m.u2 = (u.X * u.X + u.Y * u.Y) * c.inv_r2;
+  m.theta = u.th;
+  return m;
+}
+
 // ------------------------------------------------------------------------------------------
 // Kernels
 // ------------------------------------------------------------------------------------------
+
+// Pull, BGK and store of an FP64 node in fixed point; false if it is out of that range (what was
+// stored then is no result).
+template <class S, bool STREAM>
+__device__ __forceinline__ bool bgk_fixed(const Geom& g, const fx::Consts& c,
+                                          const double* __restrict__ A, double* __restrict__ B,
+                                          long long src, long long dst) {
+  fx::i64 F[S::Q];
+  if (!load_fixed<S, STREAM>(F, A, g, c, src)) return false;
+  fx::State u;
+  if (!fx::state(fx::moments<S>(F), c, u)) return false;
+  const fx::Site k = fx::site<S::ORDER>(u.X, u.Y, u.th, c.r2, c.inv_r2);
+  int low = 1;
+  each_equilibrium<S>(c, k, u.rho, [&](auto i, auto s, fx::i64 feq) {
+    B[(long long)i * g.plane + dst] =
+        fx::store(fx::relax(F[i], feq, c.om), fx::shell_fe<S>(s), c.E, low);
+  });
+  return low >= 1;
+}
 
 // Interior of F (inside the frame depths Fw, Fe, Fs, Fn): pull, moments, BGK, store.
 // Block: 32 x BY threads; the x tiles start on a 32-node boundary of F.
@@ -377,6 +454,9 @@ __device__ __forceinline__ void bulk_node(const Geom& g, const Consts<Real>& c,
                                           int* flag, int x, int y) {
   if (x < g.Fw || x >= g.Lx - g.Fe || y >= g.Ly - g.Fn) return;
   const long long idx = gindex(g, x, y);
+  if constexpr (sizeof(Real) == 8) {
+    if (c.fx.on && bgk_fixed<S, STREAM>(g, c.fx, A, B, idx, idx)) return;
+  }
   Real p[S::Q];
   load_pop<S, Real, STREAM>(p, A, g, idx);
   const Macro<Real> m = moments<S, Real, DEV>(p, c);
@@ -386,8 +466,18 @@ __device__ __forceinline__ void bulk_node(const Geom& g, const Consts<Real>& c,
   for (int i = 0; i < S::Q; ++i) B[(long long)i * g.plane + idx] = p[i];
 }
 
+// Blocks of 128 threads per SM of the FP64 interior. The fixed-point update is bound by issue and
+// by the FP64 section of its scalars, so more warps hide one behind the other until registers
+// spill. Measured at 1024^2, blocks per SM (registers): D2Q37 2 (172) 290 us, 3 (168) 237, 4 (128)
+// 215, 5 (96, spills) 264; D2Q17 4 (128) 113, 5 (96) 101; D2Q9 4 (96) 77, 8 (59) 63. FP64
+// arithmetic: 738, 385 and 203 us.
+template <class S, class Real>
+constexpr int bulk_blocks() {
+  return sizeof(Real) == 4 ? 0 : S::Q == 37 ? 4 : S::Q == 17 ? 5 : 8;   // 0: no bound
+}
+
 template <class S, class Real, bool DEV, bool STREAM>
-__global__ void __launch_bounds__(256) k_bulk(Geom g, Consts<Real> c, const Real* __restrict__ A,
+__global__ void __launch_bounds__(sizeof(Real) == 8 ? 128 : 256, bulk_blocks<S, Real>()) k_bulk(Geom g, Consts<Real> c, const Real* __restrict__ A,
                                               Real* __restrict__ B, int* flag) {
   const int x0 = (g.Fw / 32) * 32;
   bulk_node<S, Real, DEV, STREAM>(g, c, A, B, flag, x0 + blockIdx.x * 32 + threadIdx.x,

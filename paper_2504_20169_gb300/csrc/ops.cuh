@@ -222,7 +222,7 @@ struct MemberDev {
 };
 
 template <class S, class Real, bool DEV>
-__global__ void __launch_bounds__(256) kb_bulk(const MemberDev<Real>* __restrict__ mem,
+__global__ void __launch_bounds__(256, (bulk_blocks<S, Real>() + 1) / 2) kb_bulk(const MemberDev<Real>* __restrict__ mem,
                                                const int* __restrict__ tab) {
   const int* e = tab + 3 * blockIdx.x;
   const MemberDev<Real>& md = mem[e[0]];
