@@ -161,29 +161,30 @@ void mean_equilibrium(const double* w, double r, const lbm_bc_params& bp, double
 
 int halo_of(int q) { return q == 9 ? 1 : 3; }
 
-// Fixed-point constants of an FP64 context (fixed.cuh). They stay off where that arithmetic does
+// Fixed-point constants of an FP64 context (fixed.cuh), from the doubles that the FP64 arithmetic
+// multiplies by: the sums of these miss the quadrature by 1e-16, so T drifts by 3e-16 a step, and
+// both arithmetics then drift alike. They stay off where that arithmetic does
 // not apply: omega outside (0, 2), or a mean state outside its range.
 template <class S>
-void fixed_consts(const double* w, double r, double omega, const lbm_bc_params& bp,
+void fixed_consts(const double* w, double r2, double omega, const lbm_bc_params& bp,
                   const double* fbar, fx::Consts& c) {
   std::memset(&c, 0, sizeof c);
   auto units = [](long double v, int e) { return (fx::i64)std::llrint(std::ldexp(v, e)); };
-  c.r2 = r * r;
-  c.inv_r2 = 1.0 / c.r2;
+  c.r2 = fx::split(units(r2, 60));
+  c.inv_r2 = fx::split(units(1.0L / r2, 60));
   if (!(omega > 0.0) || !(omega < 2.0)) return;
   const double lg = std::log2(bp.rho0);
   if (!(std::fabs(lg) < 60.0)) return;
   c.E = (int)std::lround(lg);
-  c.om = fx::split(units(omega, 61));
-  for (int s = 0; s < S::NSHELL; ++s) {
-    const long double v = std::ldexp((long double)w[S::shell_first(s)], fx::shell_k<S>(s));
-    if (!(v > 0.5L && v < 1.0L)) return;
-    c.w[s] = fx::split(units(v, 62));
-    for (int i = S::shell_first(s); i < S::shell_first(s) + S::shell_size(s); ++i) {
-      const long double f = std::ldexp((long double)fbar[i], fx::shell_fe<S>(s) - c.E);
-      if (!(std::fabs(f) < std::ldexp(1.0L, 60))) return;
-      c.eqbar[i] = (fx::i64)std::llrint(f);
-    }
+  c.om = fx::factor(units(omega, 61));
+  if (!fx::make_shells<S>(w, c.shell)) return;
+  for (int i = 0; i < S::Q; ++i) {
+    int k = 0;
+    for (int j = 0; j < S::NSHELL; ++j)
+      if (c.shell[j].first <= i && c.shell[j].first >= c.shell[k].first) k = j;
+    const long double f = std::ldexp((long double)fbar[i], c.shell[k].fe - c.E);
+    if (!(std::fabs(f) < std::ldexp(1.0L, 59))) return;
+    c.eqbar[i] = (fx::i64)std::llrint(f);
   }
   c.on = 1;
 }
@@ -580,11 +581,36 @@ lbm_status lbm_create(const lbm_grid* grid, lbm_stencil stencil, double tau, int
   }
   d.cd.r = ctx->r; d.cd.r2 = ctx->r * ctx->r; d.cd.omega = ctx->omega;
   d.cd.sigma_max = sg.sigma_max; d.cd.power = sg.power; d.cd.split = sg.split;
-  if (q == 37) fixed_consts<D2Q37>(ctx->w, ctx->r, ctx->omega, bp, fbar, d.cd.fx);
-  else if (q == 17) fixed_consts<D2Q17>(ctx->w, ctx->r, ctx->omega, bp, fbar, d.cd.fx);
-  else fixed_consts<D2Q9>(ctx->w, ctx->r, ctx->omega, bp, fbar, d.cd.fx);
+  if (q == 37) fixed_consts<D2Q37>(ctx->w, d.cd.r2, ctx->omega, bp, fbar, d.cd.fx);
+  else if (q == 17) fixed_consts<D2Q17>(ctx->w, d.cd.r2, ctx->omega, bp, fbar, d.cd.fx);
+  else fixed_consts<D2Q9>(ctx->w, d.cd.r2, ctx->omega, bp, fbar, d.cd.fx);
   d.cf.r = (float)ctx->r; d.cf.r2 = (float)(ctx->r * ctx->r); d.cf.omega = (float)ctx->omega;
   d.cf.sigma_max = (float)sg.sigma_max; d.cf.power = sg.power; d.cf.split = sg.split;
+  {
+    // sigma of every layer of the W, E, S and N edge (index 0: none), as sigma_of forms it, in the
+    // part of the target buffer that the fused Runge-Kutta launch leaves free (12 M (Lx + Ly) or
+    // more doubles against at most Lx + Ly + 4)
+    std::vector<double> sd;
+    std::vector<float> sf;
+    for (int e = 0; e < 4; ++e)
+      for (int i = 0; i <= W4[e]; ++i) {
+        double pd = 1.0;
+        float pf = 1.0f;
+        for (int k = 0; k < sg.power; ++k) {
+          pd *= (double)i / (double)W4[e];
+          pf *= (float)i / (float)W4[e];
+        }
+        sd.push_back(i ? d.cd.sigma_max * pd : 0.0);
+        sf.push_back(i ? d.cf.sigma_max * pf : 0.0f);
+      }
+    const bool f32 = precision == LBM_FP32_DEV;
+    if (cudaMemcpyAsync(d.Va, f32 ? (const void*)sf.data() : (const void*)sd.data(),
+                        f32 ? sf.size() * sizeof(float) : sd.size() * sizeof(double),
+                        cudaMemcpyHostToDevice, ctx->st) != cudaSuccess)
+      return oom("sigma table");
+    d.cd.sigma = d.Va;
+    d.cf.sigma = reinterpret_cast<const float*>(d.Va);
+  }
   if (ctx->ops.prepare(ctx->w) != cudaSuccess) return oom("kernel attributes");
   {
     // the context's one-member plan, for buffer parity 0 and 1

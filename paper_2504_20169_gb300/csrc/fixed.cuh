@@ -3,30 +3,34 @@
 // GB300 issues one FP64 instruction per warp in 64 cycles and quadrant of an SM (76 when all four
 // quadrants do), measured; a 64-bit integer add takes 3 cycles and a 64 x 62 bit product about 20.
 // A D2Q37 update has about 390 FP64 instructions, most of them additions, so the FP64 kernels are
-// bound by that pipe at a tenth of the memory bandwidth. Here populations are exact integers from
-// load to store, and FP64 is left with the site's scalars (about 70 operations per node).
+// bound by that pipe at a tenth of the memory bandwidth. Here a node is integers from load to
+// store: populations, moments, the scalars of its equilibrium and the relaxation.
 //
-// Formats. A population of a shell with weight w is F = f 2^(fe - E), fe = 57 + k with
-// w 2^k in (1/2, 1) (two bits less on the outer shells n = |e|^2 >= 8, whose equilibrium factor
-// spans four times the range), E = the exponent of the mean density: near the state of rest one
-// unit of F is 2^-56 of the population (2^-54 on the outer shells), an eighth of the unit in the
-// last place of its double. Reading a double is exact down to a small fraction of the rest
-// population; products are rounded to nearest with the mean of their dropped low part added (no
-// bias), and the store rounds to nearest. So each population is off by less than in FP64, whose
-// equilibrium rounds several times at 2^-53.
-// The equilibrium factor P = f_eq / (w rho) is an integer polynomial in the lattice velocity with
-// the site's scalars, in units of 2^-60 (2^-58 on the outer shells).
+// Formats. A population of a shell with weight w is F = f 2^(fe - E), fe = 55 + k with
+// w 2^k in (1/2, 1), E = the exponent of the mean density: near the state of rest one unit of F is
+// 2^-54 to 2^-55 of the population, a half to a quarter of the unit in the last place of its
+// double. Reading a double of about its weight is exact; products are rounded to nearest with
+// the mean of their dropped low part added (no bias), and the store rounds to nearest. So each
+// population is off by less than in FP64, whose equilibrium rounds several times at 2^-53.
+// Velocity, temperature and what follows from them are in units of 2^-60 (FP64 has 2^-53 of the
+// value). The equilibrium factor P = f_eq / (w rho) is an integer polynomial in the lattice
+// velocity with the site's scalars, in units of 2^-58.
 //
 // Range. A node takes this path if every population is in [0, 2^59) units, 1/2 < rho 2^-E < 2,
-// |r u|^2 <= 0.7 (|u| <= 0.7 on D2Q37) and |T - 1| <= 1/4: then |P| < 8 (32 on the outer shells)
-// and no sum or product leaves its integer. Every other node (NaN and infinities too) takes the
-// FP64 arithmetic.
+// |r u|^2 <= 0.7 (|u| <= 0.7 on D2Q37) and |T - 1| <= 1/4: then |P| < 32 and no sum or product
+// leaves its integer. Every other node (NaN and infinities too) takes the FP64 arithmetic.
+//
+// Layout. A thread keeps its node in shared memory (value i at f[i * stride]) and walks the shells
+// in rolled loops, one for each of the three kinds of shell: unrolled over the directions with
+// everything in registers the code is 70 KB and misses the instruction cache, and 128 registers
+// a thread leave four warps to a scheduler.
 //
 // Host and device: everything here compiles for both, so the arithmetic can be checked on a CPU.
 #pragma once
+#include <cmath>
 #include <cstdint>
 #include <cstring>
-#include <utility>
+#include <type_traits>
 
 #include "stencils.cuh"
 
@@ -34,7 +38,6 @@
 #define LBM_HD __host__ __device__ __forceinline__
 #else
 #define LBM_HD inline
-#include <cmath>
 #endif
 
 namespace lbm {
@@ -42,16 +45,6 @@ namespace fx {
 
 typedef long long i64;
 typedef unsigned long long u64;
-
-// fn(integral_constant<0>) ... fn(integral_constant<N - 1>): arrays indexed inside stay in registers
-template <class Fn, int... I>
-LBM_HD void unroll_seq(Fn&& fn, std::integer_sequence<int, I...>) {
-  (fn(std::integral_constant<int, I>()), ...);
-}
-template <int N, class Fn>
-LBM_HD void unroll(Fn&& fn) {
-  unroll_seq(fn, std::make_integer_sequence<int, N>());
-}
 
 LBM_HD u64 bits_of(double v) {
 #ifdef __CUDA_ARCH__
@@ -85,6 +78,8 @@ LBM_HD int clz32(unsigned v) {
   return v ? __builtin_clz(v) : 32;
 #endif
 }
+// 2^e, -1022 <= e <= 1023
+LBM_HD double pow2(int e) { return double_of((u64)(unsigned)(1023 + e) << 52); }
 // v >> s for s >= 0, zero from 64 on
 LBM_HD u64 shr(u64 v, int s) {
 #ifdef __CUDA_ARCH__
@@ -105,52 +100,60 @@ LBM_HD u64 shl(u64 v, int s) {
 #endif
 }
 
-// A factor 0 <= v < 2^62 as two 32-bit limbs, v = h 2^32 + l with l signed, so that every
-// partial product with a 64-bit integer is one native 32 x 32 -> 64 bit multiplication.
+// A factor |v| < 2^63 as two signed 32-bit limbs, v = h 2^32 + l: every partial product is one
+// native 32 x 32 -> 64 bit multiplication.
 struct Limbs {
-  unsigned h;
-  int l;
+  int h, l;
 };
 LBM_HD Limbs split(i64 v) {
   const u64 r = (u64)v + 0x80000000u;
-  return Limbs{(unsigned)(r >> 32), (int)(unsigned)v};
+  return Limbs{(int)(r >> 32), (int)(unsigned)v};
 }
 
-// a b / 2^64, off by less than one unit and by none on average: the product of the low limbs
-// (mean 0, as l is signed) is left out, and 2^31 rounds.
-LBM_HD i64 mul(i64 a, Limbs b) {
+// A factor 0 <= v < 2^62 of many products: its limbs and the constant that rounds them.
+struct Factor {
+  int h, l;
+  unsigned c;        // 2^31 + l / 2
+};
+LBM_HD Factor factor(i64 v) {
+  const Limbs b = split(v);
+  return Factor{b.h, b.l, 0x80000000u + (unsigned)(b.l >> 1)};
+}
+
+// a b / 2^64, off by less than one unit and by none on average: the product of the low limbs is
+// replaced by its mean over the low limb of a, and 2^31 rounds.
+LBM_HD i64 mul(i64 a, Factor b) {
   const int ah = (int)(a >> 32);
-  i64 m = (i64)ah * b.l + (1ll << 31);
-  m += (i64)((u64)(unsigned)a * b.h);
-  return (i64)ah * (int)b.h + (m >> 32);
+  i64 m = (i64)ah * b.l + (i64)(u64)b.c;
+  m += (i64)((u64)(unsigned)a * (unsigned)b.h);
+  return (i64)ah * b.h + (m >> 32);
 }
 
-// Weight exponent of a shell: w 2^k in (1/2, 1) (checked when a context is created).
+// a b in units of 2^-TO for a, b in units of 2^-60 (|a| + |b| < 16), off by 2^(TO - 58) at most.
+template <int TO = 60>
+LBM_HD i64 prod(Limbs a, Limbs b) {
+  constexpr int up = TO - 56;
+  i64 m = (i64)a.h * b.l + (1ll << (31 - up));
+  m += (i64)a.l * b.h;
+  return (i64)((u64)((i64)a.h * b.h) << up) + (m >> (32 - up));
+}
+
+// A shell as the loops see it: velocities of base (a, b), a >= b, from direction `first` on.
+struct ShellInfo {
+  int first, a, b, fe;
+  Factor w;          // weight w 2^k in units of 2^-62
+};
+
+// Kinds of shell: (0, 0), then (a, 0), then (a, a), then (a, b).
 template <class S>
-LBM_HD constexpr int shell_k(int s) {
-  if (S::Q == 37) {
-    constexpr int t[8] = {2, 3, 4, 6, 7, 9, 11, 11};
-    return t[s];
-  }
-  if (S::Q == 17) {
-    constexpr int t[8] = {1, 3, 4, 13, 11, 0, 0, 0};
-    return t[s];
-  }
-  constexpr int t[8] = {1, 3, 5, 0, 0, 0, 0, 0};
-  return t[s];
+LBM_HD constexpr int kind_of(int s) {
+  return S::shell_a(s) == 0 ? 0 : S::shell_b(s) == 0 ? 1 : S::shell_a(s) == S::shell_b(s) ? 2 : 3;
 }
 template <class S>
-LBM_HD constexpr int shell_n(int s) {
-  return S::shell_a(s) * S::shell_a(s) + S::shell_b(s) * S::shell_b(s);
-}
-// bits by which an outer shell is coarser
-template <class S>
-LBM_HD constexpr int shell_far(int s) {
-  return shell_n<S>(s) >= 8 ? 2 : 0;
-}
-template <class S>
-LBM_HD constexpr int shell_fe(int s) {
-  return 57 + shell_k<S>(s) - shell_far<S>(s);
+LBM_HD constexpr int kind_count(int kind) {
+  int n = 0;
+  for (int s = 0; s < S::NSHELL; ++s) n += kind_of<S>(s) == kind ? 1 : 0;
+  return n;
 }
 
 // f 2^(fe - E) of a double f >= 0. `low` takes the smallest right shift seen: below 3 a
@@ -164,6 +167,10 @@ LBM_HD i64 load(double f, int fe, int E, int& low) {
   return (i64)shr(m, s < 0 ? 0 : s);
 }
 
+// The leading 53 bits of a value with its top bit at 62, to nearest, halves to even (with two to
+// four bits to drop, halves are common); a carry moves the exponent up where it is added.
+LBM_HD u64 round53(u64 n) { return (n + 0x1ff + ((unsigned)(n >> 10) & 1u)) >> 10; }
+
 // The double nearest to F 2^(E - fe) for 2^32 <= F < 2^62; `low` takes the smallest upper word
 // seen: below 1 a value is out of this range (a population that is negative or 2^-25 of its
 // weight) and the result is not the value.
@@ -171,7 +178,7 @@ LBM_HD double store(i64 F, int fe, int E, int& low) {
   const int fh = (int)(F >> 32);
   low = fh < low ? fh : low;
   const int z = clz32((unsigned)fh);
-  const u64 r = (shl((u64)F, z - 1) + 0x200) >> 10;   // 53 bits, rounded; a carry moves the exponent up
+  const u64 r = round53(shl((u64)F, z - 1));
   const unsigned hi = (unsigned)(r >> 32) + ((unsigned)(1023 + 62 - fe + E - z) << 20);
   return double_of((u64)hi << 32 | (unsigned)r);
 }
@@ -180,14 +187,14 @@ LBM_HD double store(i64 F, int fe, int E) {
   const i64 sg = F >> 63;
   const u64 m = (u64)((F ^ sg) - sg);
   const int z = clz(m);
-  const u64 r = (shl(m, z - 1) + 0x200) >> 10;
+  const u64 r = round53(shl(m, z - 1));
   const unsigned hi = (unsigned)(r >> 32) + ((unsigned)(1023 + 62 - fe + E - z) << 20) +
                       ((unsigned)(F >> 32) & 0x80000000u);
   return m ? double_of((u64)hi << 32 | (unsigned)r) : 0.0;
 }
 
-// A site scalar |v| < 8 in units of 2^-60, truncated.
-LBM_HD i64 scalar(double v) {
+// |v| < 8 in units of 2^-60, truncated.
+LBM_HD i64 fixed60(double v) {
   const u64 b = bits_of(v);
   const unsigned hi = (unsigned)(b >> 32);
   const u64 m = (((u64)((hi & 0xfffffu) | 0x100000u)) << 32 | (unsigned)b) << 10;   // top bit 62
@@ -196,11 +203,12 @@ LBM_HD i64 scalar(double v) {
   return (a ^ sg) - sg;
 }
 
-// Constants of a context: the shells' weights w 2^k in units of 2^-62, the relaxation rate in
-// units of 2^-61, the exponent E, and the mean equilibrium in each direction's units.
+// Constants of a context: the shells ordered by kind, the relaxation rate in units of 2^-61, the
+// exponent E, and the mean equilibrium in each direction's units.
 struct Consts {
-  Limbs w[8], om;
-  double r2, inv_r2;
+  ShellInfo shell[8];
+  Factor om;
+  Limbs r2, inv_r2;  // r^2 and 1 / r^2 in units of 2^-60
   int E;
   int on;          // 0: FP64 arithmetic everywhere (omega = 0 keeps populations bit for bit)
   i64 eqbar[37];
@@ -215,194 +223,297 @@ struct Site {
   i64 A0, A1, A2, B, P0, P1, Q0, Q1, Q2, Rx0, Rx1, Tx, Ry0, Ry1, Ty;
 };
 
-// X = r u_x, Y = r u_y, theta = T - 1. |X|^2 + |Y|^2 <= 0.7 and |theta| <= 1/4 keep every
-// scalar below 4.
+// Macroscopic state of a node in range.
+struct State {
+  i64 rho;           // rho 2^-E in units of 2^-58
+  i64 X, Y, th;      // r u and T - 1 in units of 2^-60
+};
+
+// v / 4, to nearest, halves to even: rounding these scalars down would lose 1e-17 of rho and T in
+// every step.
+LBM_HD i64 quarter(i64 v) { return (v + 1 + ((unsigned)(v >> 2) & 1u)) >> 2; }
+
+// From the state: |X|^2 + |Y|^2 <= 0.7 and |theta| <= 1/4 keep every value here below 4.
 template <int ORDER>
-LBM_HD Site site(double X, double Y, double th, double r2, double inv_r2) {
-  const double p = X * X, m = Y * Y, xy = X * Y, S = p + m, D = p - m;
-  const double u2 = S * inv_r2, rt = r2 * th;
+LBM_HD Site site(const State& u, const Consts& c) {
+  const i64 ONE = 1ll << 60;
+  const Limbs X = split(u.X), Y = split(u.Y), th = split(u.th);
+  const i64 p = prod(X, X), m = prod(Y, Y), xy = prod(X, Y), S = p + m, D = p - m;
+  const Limbs Ss = split(S), Ds = split(D), xs = split(xy);
+  const i64 u2 = prod(Ss, c.inv_r2), rt = prod(c.r2, th);
+  const i64 one = ONE - (u2 >> 1);
+  // 1/48, 1/12 and 1/6 in units of 2^-60
+  const Limbs k48 = split(ONE / 48), k12 = split(ONE / 12), k6 = split(ONE / 6);
   Site k;
   k.A2 = k.B = k.P1 = k.Q1 = k.Q2 = k.Rx1 = k.Tx = k.Ry1 = k.Ty = 0;
-  const double one = 1.0 - 0.5 * u2;
   if (ORDER >= 4) {
-    const double half = 0.5 - 0.25 * u2;
-    const double k20 = half - 1.5 * th;
-    const double x4 = S * S - 2.0 * (p * m);
-    const double z = S * (1.0 / 48.0) + 0.125 * rt;
-    k.A0 = scalar((one - th) + th * (th + u2) + 0.125 * (u2 * u2));
-    k.A1 = scalar(rt * (half - th) + 0.5 * (k20 * S));
-    k.A2 = scalar(0.125 * (rt * (rt + S)) + x4 * (1.0 / 48.0));
-    k.B = scalar(0.25 * (p * m) - x4 * (1.0 / 24.0));
-    k.P0 = scalar(0.5 * (k20 * D));
-    k.P1 = scalar(z * D);
-    k.Q0 = scalar(2.0 * (xy * k20));
-    k.Q1 = scalar(4.0 * (xy * z));
-    k.Q2 = scalar(xy * (D * (1.0 / 12.0)));
+    const i64 half = (ONE >> 1) - (u2 >> 2);
+    const Limbs k20 = split(half - u.th - (u.th >> 1)), rs = split(rt), us = split(u2);
+    const i64 pm = prod(xs, xs), x48 = prod(split(prod(Ss, Ss) - 2 * pm), k48);
+    const Limbs t = split(S + 6 * rt);
+    k.A0 = quarter(one - u.th + prod(th, split(u.th + u2)) + (prod(us, us) >> 3));
+    k.A1 = quarter(prod(rs, split(half - u.th)) + (prod(k20, Ss) >> 1));
+    k.A2 = quarter((prod(rs, split(rt + S)) >> 3) + x48);
+    k.B = quarter((pm >> 2) - 2 * x48);
+    const Limbs x12 = split(prod(xs, k12));
+    k.P0 = prod<57>(k20, Ds);
+    k.P1 = prod<58>(t, split(prod(Ds, k48)));
+    k.Q0 = prod<59>(xs, k20);
+    k.Q1 = prod<58>(t, x12);
+    k.Q2 = prod<58>(Ds, x12);
   } else {
-    k.A0 = scalar(one - th);
-    k.A1 = scalar(0.5 * rt + 0.25 * S);
-    k.P0 = scalar(0.25 * D);
-    k.Q0 = scalar(xy);
+    k.A0 = quarter(one - u.th);
+    k.A1 = quarter((rt >> 1) + (S >> 2));
+    k.P0 = D >> 4;
+    k.Q0 = quarter(xy);
   }
   if (ORDER >= 3) {
-    const double k10 = one - 2.0 * th;
-    k.Rx0 = scalar(X * k10);
-    k.Ry0 = scalar(Y * k10);
-    k.Rx1 = scalar(0.5 * (X * (rt + m)));
-    k.Ry1 = scalar(0.5 * (Y * (rt + p)));
-    k.Tx = scalar((X * (1.0 / 6.0)) * (p - 3.0 * m));
-    k.Ty = scalar((Y * (1.0 / 6.0)) * (m - 3.0 * p));
+    const Limbs k10 = split(one - 2 * u.th);
+    k.Rx0 = prod<58>(X, k10);
+    k.Ry0 = prod<58>(Y, k10);
+    k.Rx1 = prod<57>(X, split(rt + m));
+    k.Ry1 = prod<57>(Y, split(rt + p));
+    k.Tx = prod<58>(X, split(prod(split(p - 3 * m), k6)));
+    k.Ty = prod<58>(Y, split(prod(split(m - 3 * p), k6)));
   } else {
-    k.Rx0 = scalar(X);
-    k.Ry0 = scalar(Y);
+    k.Rx0 = quarter(u.X);
+    k.Ry0 = quarter(u.Y);
   }
   return k;
 }
 
-// The scalars in the outer shells' units.
-template <int ORDER>
-LBM_HD Site coarse(const Site& k) {
-  Site c;
-  c.A0 = k.A0 >> 2; c.A1 = k.A1 >> 2; c.P0 = k.P0 >> 2; c.Q0 = k.Q0 >> 2;
-  c.Rx0 = k.Rx0 >> 2; c.Ry0 = k.Ry0 >> 2;
-  c.A2 = c.B = c.P1 = c.Q1 = c.Q2 = c.Rx1 = c.Tx = c.Ry1 = c.Ty = 0;
-  if (ORDER >= 4) {
-    c.A2 = k.A2 >> 2; c.B = k.B >> 2; c.P1 = k.P1 >> 2; c.Q1 = k.Q1 >> 2; c.Q2 = k.Q2 >> 2;
-  }
-  if (ORDER >= 3) {
-    c.Rx1 = k.Rx1 >> 2; c.Tx = k.Tx >> 2; c.Ry1 = k.Ry1 >> 2; c.Ty = k.Ty >> 2;
-  }
-  return c;
-}
-
-// What the directions of a shell (a, b) share; a direction with |e_x| = a is of kind 0, with
-// |e_x| = b of kind 1 (the axes swapped).
-struct Shell {
-  i64 even[2];       // symmetric in both components
-  i64 cross[2];      // times the sign of e_x e_y
-  i64 x[2], y[2];    // times the sign of e_x, of e_y
-};
-template <class S>
-LBM_HD Shell shell(const Site& k, int s) {
-  const int a = S::shell_a(s), b = S::shell_b(s), n = a * a + b * b, d = a * a - b * b;
-  Shell h;
-  i64 sym = k.A0 + n * k.A1, anti = k.P0, q = k.Q0, ux = k.Rx0, uy = k.Ry0;
-  if (S::ORDER >= 4) {
-    sym += (n * n) * k.A2 + (a * a * b * b) * k.B;
-    anti += n * k.P1;
-    q += n * k.Q1;
-  }
-  if (S::ORDER >= 3) {
-    ux += n * k.Rx1;
-    uy += n * k.Ry1;
-  }
-  h.even[0] = sym + d * anti;
-  h.even[1] = sym - d * anti;
-  const i64 q0 = (a * b) * q, q2 = S::ORDER >= 4 ? (a * b * d) * k.Q2 : 0;
-  h.cross[0] = q0 + q2;
-  h.cross[1] = q0 - q2;
-  h.x[0] = a * ux;
-  h.x[1] = b * ux;
-  h.y[0] = b * uy;
-  h.y[1] = a * uy;
-  if (S::ORDER >= 3) {
-    h.x[0] += (a * a * a) * k.Tx;
-    h.x[1] += (b * b * b) * k.Tx;
-    h.y[0] += (b * b * b) * k.Ty;
-    h.y[1] += (a * a * a) * k.Ty;
-  }
-  return h;
-}
-// Even and odd part of P of one direction of the shell.
-template <class S>
-LBM_HD void factor(const Shell& h, int s, int ex, int ey, i64& even, i64& odd) {
-  const int kind = (ex < 0 ? -ex : ex) == S::shell_a(s) ? 0 : 1;
-  even = h.even[kind];
-  if (ex * ey > 0) even += h.cross[kind];
-  if (ex * ey < 0) even -= h.cross[kind];
-  odd = ex > 0 ? h.x[kind] : ex < 0 ? -h.x[kind] : 0;
-  if (ey > 0) odd += h.y[kind];
-  if (ey < 0) odd -= h.y[kind];
-}
-
 // The weight of a shell times the density (rho 2^-E in units of 2^-58), in units of 2^-61: the
 // second factor of every direction's equilibrium, below 2^62.
-template <class S>
-LBM_HD Limbs shell_weight(const Consts& c, int s, i64 rho58) {
-  return split(2 * mul(rho58 << 4, c.w[s]));
-}
-
-// f_eq in the direction's units from P (units of 2^-60, on the outer shells 2^-58).
-LBM_HD i64 equilibrium(i64 P, Limbs wr) { return mul(P, wr); }
+LBM_HD Factor shell_weight(const ShellInfo& h, i64 rho58) { return factor(2 * mul(rho58 << 4, h.w)); }
 
 // F + omega (feq - F); |feq - F| < 2^60.
-LBM_HD i64 relax(i64 F, i64 feq, Limbs om) { return F + mul((feq - F) * 8, om); }
+LBM_HD i64 relax(i64 F, i64 feq, Factor om) { return F + mul((feq - F) * 8, om); }
+
+// put(h, shell, feq) for every direction shell.first + h with its equilibrium in fixed point;
+// pre(shell, size) before a shell (h and size are integral constants).
+template <class S, class Pre, class Put>
+LBM_HD void each_equilibrium(const Consts& c, const Site& k, i64 rho58, Pre pre, Put put) {
+  constexpr int axis = kind_count<S>(1), diag = kind_count<S>(2), octet = kind_count<S>(3);
+  using std::integral_constant;
+  integral_constant<int, 0> h0;
+  integral_constant<int, 1> h1;
+  integral_constant<int, 2> h2;
+  integral_constant<int, 3> h3;
+  integral_constant<int, 4> h4;
+  integral_constant<int, 5> h5;
+  integral_constant<int, 6> h6;
+  integral_constant<int, 7> h7;
+  integral_constant<int, 8> h8;
+  {
+    const ShellInfo& h = c.shell[0];
+    pre(h, h1);
+    put(h0, h, mul(k.A0, shell_weight(h, rho58)));
+  }
+#pragma unroll 1
+  for (int j = 0; j < axis; ++j) {
+    const ShellInfo& h = c.shell[1 + j];
+    pre(h, h4);
+    const Factor w = shell_weight(h, rho58);
+    const int a = h.a, n = a * a;
+    i64 sym = k.A0 + n * k.A1, anti = k.P0, x = k.Rx0, y = k.Ry0;
+    if (S::ORDER >= 4) {
+      sym += (n * n) * k.A2;
+      anti += n * k.P1;
+    }
+    if (S::ORDER >= 3) {
+      x += n * (k.Rx1 + k.Tx);
+      y += n * (k.Ry1 + k.Ty);
+    }
+    x *= a;
+    y *= a;
+    anti *= n;
+    put(h0, h, mul(sym + anti + x, w));
+    put(h1, h, mul(sym - anti + y, w));
+    put(h2, h, mul(sym + anti - x, w));
+    put(h3, h, mul(sym - anti - y, w));
+  }
+#pragma unroll 1
+  for (int j = 0; j < diag; ++j) {
+    const ShellInfo& h = c.shell[1 + axis + j];
+    pre(h, h4);
+    const Factor w = shell_weight(h, rho58);
+    const int a = h.a, a2 = a * a, n = 2 * a2;
+    i64 sym = k.A0 + n * k.A1, cross = k.Q0, x = k.Rx0, y = k.Ry0;
+    if (S::ORDER >= 4) {
+      sym += (n * n) * k.A2 + (a2 * a2) * k.B;
+      cross += n * k.Q1;
+    }
+    if (S::ORDER >= 3) {
+      x += n * k.Rx1 + a2 * k.Tx;
+      y += n * k.Ry1 + a2 * k.Ty;
+    }
+    cross *= a2;
+    x *= a;
+    y *= a;
+    const i64 p = sym + cross, m = sym - cross, u = x + y, v = y - x;
+    put(h0, h, mul(p + u, w));
+    put(h1, h, mul(m + v, w));
+    put(h2, h, mul(p - u, w));
+    put(h3, h, mul(m - v, w));
+  }
+#pragma unroll 1
+  for (int j = 0; j < octet; ++j) {
+    const ShellInfo& h = c.shell[1 + axis + diag + j];
+    pre(h, h8);
+    const Factor w = shell_weight(h, rho58);
+    const int a = h.a, b = h.b, a2 = a * a, b2 = b * b, ab = a * b, n = a2 + b2, d = a2 - b2;
+    const i64 sym = k.A0 + n * k.A1 + (n * n) * k.A2 + (ab * ab) * k.B;
+    const i64 anti = d * (k.P0 + n * k.P1), q = ab * (k.Q0 + n * k.Q1), q2 = (ab * d) * k.Q2;
+    const i64 ux = k.Rx0 + n * k.Rx1, uy = k.Ry0 + n * k.Ry1;
+    {   // |e_x| = a, |e_y| = b: directions 0 and 3 and their opposites 4 and 7
+      const i64 x = a * (ux + a2 * k.Tx), y = b * (uy + b2 * k.Ty);
+      const i64 p = sym + anti + q + q2, m = sym + anti - q - q2;
+      put(h0, h, mul(p + x + y, w));
+      put(h3, h, mul(m - x + y, w));
+      put(h4, h, mul(p - x - y, w));
+      put(h7, h, mul(m + x - y, w));
+    }
+    {   // |e_x| = b, |e_y| = a: 1, 2 and 5, 6
+      const i64 x = b * (ux + b2 * k.Tx), y = a * (uy + a2 * k.Ty);
+      const i64 p = sym - anti + q - q2, m = sym - anti - q + q2;
+      put(h1, h, mul(p + x + y, w));
+      put(h2, h, mul(m - x + y, w));
+      put(h5, h, mul(p - x - y, w));
+      put(h6, h, mul(m + x - y, w));
+    }
+  }
+}
+
+// Lattice velocity of direction `first + h` of a shell (for the few nodes that need it).
+LBM_HD void velocity(const ShellInfo& s, int h, int& ex, int& ey) {
+  const int a = s.a, b = s.b;
+  if (a == 0) {
+    ex = ey = 0;
+  } else if (b == 0) {
+    ex = h == 0 ? a : h == 2 ? -a : 0;
+    ey = h == 1 ? a : h == 3 ? -a : 0;
+  } else if (a == b) {
+    ex = h == 0 || h == 3 ? a : -a;
+    ey = h < 2 ? a : -a;
+  } else {
+    const int kx = h == 0 || h == 3 || h == 4 || h == 7 ? a : b;
+    ex = h < 2 || h > 5 ? kx : -kx;
+    ey = h < 4 ? a + b - kx : -(a + b - kx);
+  }
+}
 
 // Moments of a node's populations: rho, sum f e_x, sum f e_y, sum f |e|^2 (times 2^-E), in
 // units of 2^-58. Each shell is summed exactly (at most eight values below 2^59) and then
-// rounded to the common unit.
+// rounded to the common unit, which the shells up to weight 2^-4 are multiples of near rest (a
+// half rounds up: the fewer halves, the less bias).
 struct Moments {
   i64 rho, jx, jy, e2;
 };
+
+// Reads a node's doubles at f[i * stride], leaves their integers there and sums them; `low` as in
+// load().
 template <class S>
-LBM_HD Moments moments(const i64 (&F)[S::Q]) {
+LBM_HD Moments gather(const Consts& c, double* f, int stride, int& low) {
+  constexpr int axis = kind_count<S>(1), diag = kind_count<S>(2), octet = kind_count<S>(3);
+  auto get = [&](const ShellInfo& s, int h) {
+    double* at = f + (s.first + h) * stride;
+    const i64 F = load(*at, s.fe, c.E, low);
+    *at = double_of((u64)F);
+    return F;
+  };
   Moments m{0, 0, 0, 0};
-  unroll<S::NSHELL>([&](auto sc) {
-    constexpr int s = sc, i0 = S::shell_first(s), size = S::shell_size(s);
-    constexpr int sh = shell_fe<S>(s) - 58;
-    constexpr i64 half = (1ll << sh) >> 1;
-    if constexpr (size == 1) {
-      m.rho += (F[i0] + half) >> sh;
-    } else {
-      i64 sum = half, x = half, y = half;
-      unroll<size / 2>([&](auto h) {
-        constexpr int ip = i0 + h, im = ip + size / 2;
-        const i64 a = F[ip], b = F[im];
-        sum += a + b;
-        x += S::ex(ip) * (a - b);
-        y += S::ey(ip) * (a - b);
-      });
-      sum >>= sh;
-      m.rho += sum;
-      m.jx += x >> sh;
-      m.jy += y >> sh;
-      m.e2 += shell_n<S>(s) * sum;
-    }
-  });
+  auto add = [&](const ShellInfo& s, int n, i64 sum, i64 x, i64 y) {
+    const int sh = s.fe - 58;
+    const i64 half = (1ll << sh) >> 1;
+    sum = (sum + half) >> sh;
+    m.rho += sum;
+    m.jx += (x + half) >> sh;
+    m.jy += (y + half) >> sh;
+    m.e2 += n * sum;
+  };
+  {
+    const ShellInfo& s = c.shell[0];
+    m.rho = get(s, 0) << (58 - s.fe);   // the rest weight is above 1/8: fe = 56 or 57
+  }
+#pragma unroll 1
+  for (int j = 0; j < axis; ++j) {
+    const ShellInfo& s = c.shell[1 + j];
+    const i64 p0 = get(s, 0), p1 = get(s, 1), p2 = get(s, 2), p3 = get(s, 3);
+    add(s, s.a * s.a, p0 + p1 + p2 + p3, s.a * (p0 - p2), s.a * (p1 - p3));
+  }
+#pragma unroll 1
+  for (int j = 0; j < diag; ++j) {
+    const ShellInfo& s = c.shell[1 + axis + j];
+    const i64 p0 = get(s, 0), p1 = get(s, 1), p2 = get(s, 2), p3 = get(s, 3);
+    add(s, 2 * s.a * s.a, p0 + p1 + p2 + p3, s.a * (p0 - p1 - p2 + p3), s.a * (p0 + p1 - p2 - p3));
+  }
+#pragma unroll 1
+  for (int j = 0; j < octet; ++j) {
+    const ShellInfo& s = c.shell[1 + axis + diag + j];
+    const i64 p0 = get(s, 0), p1 = get(s, 1), p2 = get(s, 2), p3 = get(s, 3);
+    const i64 p4 = get(s, 4), p5 = get(s, 5), p6 = get(s, 6), p7 = get(s, 7);
+    const i64 d0 = p0 - p4, d1 = p1 - p5, d2 = p2 - p6, d3 = p3 - p7;
+    add(s, s.a * s.a + s.b * s.b, ((p0 + p1) + (p2 + p3)) + ((p4 + p5) + (p6 + p7)),
+        s.a * (d0 - d3) + s.b * (d1 - d2), s.b * (d0 + d3) + s.a * (d1 + d2));
+  }
   return m;
 }
 
-// 1 / v for v in (2^57, 2^59): Newton's iteration from the single-precision reciprocal of the
-// leading bits (conversions to and from FP64 run in the FP64 pipe: the seed avoids them).
-LBM_HD double reciprocal(i64 v) {
-  const float f = 1.0f / (float)(int)(v >> 28);
-  unsigned fb;
+// 1 / v for 1/2 < v < 2, both in units of 2^-60: from the single-precision reciprocal x of the
+// leading bits, x (1 + e + e^2) with e = 1 - v x (the geometric series; e^3 < 2^-63 is left out).
+LBM_HD i64 reciprocal(i64 v) {
+  constexpr float kScale = 72057594037927936.0f;   // 2^56
 #ifdef __CUDA_ARCH__
-  fb = __float_as_uint(f);
+  const float f = __fdividef(kScale, (float)(int)(v >> 32));
 #else
-  std::memcpy(&fb, &f, 4);
+  const float f = kScale / (float)(int)(v >> 32);
 #endif
-  const double x0 = double_of(((u64)fb << 29) + ((u64)(1023 - 127 - 28) << 52)), d = (double)v;
-  const double x1 = fma(x0, fma(-d, x0, 1.0), x0);
-  return fma(x1, fma(-d, x1, 1.0), x1);
+  const Limbs x = split((i64)(int)f << 32);
+  const i64 e = (1ll << 60) - prod(split(v), x);
+  const Limbs es = split(e);
+  return ((i64)x.h << 32) + prod(x, split(e + prod(es, es)));
 }
 
-// Macroscopic state of a node in range.
-struct State {
-  i64 rho;            // units of 2^-58, times 2^-E
-  double X, Y, th;    // r u and T - 1
-};
+// The shells of a stencil for given weights (w: one per direction); false if one lies outside the
+// weights' range.
+template <class S>
+inline bool make_shells(const double* w, ShellInfo (&out)[8]) {
+  int n = 0;
+  for (int kind = 0; kind < 4; ++kind)
+    for (int s = 0; s < S::NSHELL; ++s) {
+      if (kind_of<S>(s) != kind) continue;
+      int e;
+      const double m = std::frexp(w[S::shell_first(s)], &e);   // w = m 2^e, m in [1/2, 1)
+      if (!(m > 0.5) || e > 0 || e < -40) return false;
+      out[n++] = ShellInfo{S::shell_first(s), S::shell_a(s), S::shell_b(s), 55 - e,
+                           factor((i64)std::ldexp(m, 62))};
+    }
+  return true;
+}
+
+// 1/2 < rho 2^-E < 2, |(X, Y)|^2 <= 0.7, |T - 1| <= 1/4, for components and T - 1 known to be
+// below 2
+LBM_HD bool in_range(const State& u) {
+  const i64 top = (i64)(0.7 * (double)(1ll << 60)), quarter = 1ll << 58;
+  const Limbs X = split(u.X), Y = split(u.Y);
+  return u.rho > (1ll << 57) && u.rho < (1ll << 59) && prod(X, X) + prod(Y, Y) <= top &&
+         u.th <= quarter && u.th >= -quarter;
+}
 
 LBM_HD bool state(const Moments& m, const Consts& c, State& u) {
-  if (m.rho <= (1ll << 57) || m.rho >= (1ll << 59)) return false;
-  const double inv = reciprocal(m.rho), ri = c.r2 * inv;
+  // |sum f e| < rho and sum f |e|^2 < 4 rho hold well beyond the range and keep the quotients small
+  if (m.rho <= (1ll << 57) || m.rho >= (1ll << 59) || m.jx >= m.rho || -m.jx >= m.rho ||
+      m.jy >= m.rho || -m.jy >= m.rho || m.e2 >= 4 * m.rho)
+    return false;
+  const Limbs ri = split(prod(c.r2, split(reciprocal(m.rho << 2))));
   u.rho = m.rho;
-  u.X = (double)m.jx * ri;
-  u.Y = (double)m.jy * ri;
+  u.X = prod(split(m.jx << 2), ri);
+  u.Y = prod(split(m.jy << 2), ri);
   // D rho T = r^2 sum f |e|^2 - rho u^2 with D = 2 and u = (X, Y) / r
-  const double s = u.X * u.X + u.Y * u.Y;
-  u.th = 0.5 * ((double)m.e2 * ri - s * c.inv_r2) - 1.0;
-  return s <= 0.7 && u.th <= 0.25 && u.th >= -0.25;
+  const Limbs X = split(u.X), Y = split(u.Y);
+  const i64 u2 = prod(split(prod(X, X) + prod(Y, Y)), c.inv_r2);
+  u.th = prod(split(m.e2 << 1), ri) - (u2 >> 1) - (1ll << 60);
+  return in_range(u);
 }
 
 }  // namespace fx

@@ -70,6 +70,7 @@ struct Consts : FixedConsts<Real> {
   Real r, r2, omega, sigma_max;
   int power;
   int split;         // 1: sigma_x != sigma_y (Eq. pml-general), 0: sigma_x = sigma_y (Eq. PMLCOLL)
+  const Real* sigma; // sigma of the layers 0 .. W of the W, E, S and N edge, one after the other
 };
 
 struct BcParams {
@@ -164,6 +165,30 @@ __device__ inline void pml_sigmas(const Consts<Real>& c, const PmlNode<Real>& n,
     sx = sigma_of(c, n.fx > n.fy ? n.fx : n.fy);
     sy = sx;
   }
+}
+
+// The same from the table of the layers' sigma (the same values: the larger fraction has the
+// larger sigma), without the divisions and the power: 20 to 30 FP64 operations per node.
+template <class Real>
+struct PmlLayers {
+  bool has_q, in_p;
+  Real sx, sy;
+};
+template <class Real>
+__device__ inline PmlLayers<Real> pml_layers(const Geom& g, const Consts<Real>& c, int x, int y) {
+  const int ex = g.Lx - 1 - x, ey = g.Ly - 1 - y;
+  const int iw = max(0, g.Ww - x), ie = max(0, g.We - ex);
+  const int is = max(0, g.Ws - y), in = max(0, g.Wn - ey);
+  PmlLayers<Real> n;
+  n.in_p = (iw | ie | is | in) > 0;
+  const int r = g.qr - 1;
+  n.has_q = (g.Ww > 0 && x <= g.Ww + r) || (g.We > 0 && ex <= g.We + r) ||
+            (g.Ws > 0 && y <= g.Ws + r) || (g.Wn > 0 && ey <= g.Wn + r);
+  const int e = g.Ww + 1, s = e + g.We + 1, t = s + g.Ws + 1;
+  n.sx = iw > 0 ? __ldg(c.sigma + iw) : ie > 0 ? __ldg(c.sigma + e + ie) : Real(0);
+  n.sy = is > 0 ? __ldg(c.sigma + s + is) : in > 0 ? __ldg(c.sigma + t + in) : Real(0);
+  if (!c.split) n.sx = n.sy = n.sx > n.sy ? n.sx : n.sy;
+  return n;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -371,54 +396,48 @@ __device__ inline void load_pop(Real (&p)[S::Q], const Real* __restrict__ A, con
   }
 }
 
-// Populations of an FP64 node as fixed-point integers; false if one is out of their range.
-template <class S, bool STREAM>
-__device__ __forceinline__ bool load_fixed(fx::i64 (&F)[S::Q], const double* __restrict__ A,
-                                           const Geom& g, const fx::Consts& c, long long idx) {
-  int low = 1 << 20;
-  fx::unroll<S::NSHELL>([&](auto s) {
-    fx::unroll<S::shell_size(s)>([&](auto h) {
-      constexpr int i = S::shell_first(s) + h;
-      const long long src = STREAM ? pull_src(g, idx, S::ex(i), S::ey(i)) : idx;
-      F[i] = fx::load(__ldg(A + (long long)i * g.plane + src), fx::shell_fe<S>(s), c.E, low);
-    });
-  });
-  return low >= 3;
+// 4- and 8-byte asynchronous global -> shared copies (cp.async) and the wait for all of this
+// thread's copies.
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(double* dst, const double* src) {
+  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
 }
 
-// put(i, s, feq) for every direction i (of shell s; both integral constants) with its
-// equilibrium in fixed point.
-template <class S, class Put>
-__device__ __forceinline__ void each_equilibrium(const fx::Consts& c, const fx::Site& k,
-                                                 fx::i64 rho58, Put put) {
-  fx::unroll<S::NSHELL>([&](auto s) {
-    constexpr int i0 = S::shell_first(s), n = S::shell_size(s);
-    const fx::Limbs wr = fx::shell_weight<S>(c, s, rho58);
-    if constexpr (n == 1) {
-      put(std::integral_constant<int, i0>(), s, fx::equilibrium(k.A0, wr));
-    } else {
-      const fx::Shell sh = fx::shell<S>(fx::shell_far<S>(s) ? fx::coarse<S::ORDER>(k) : k, s);
-      fx::unroll<n / 2>([&](auto h) {
-        constexpr int ip = i0 + h, im = ip + n / 2;
-        fx::i64 even, odd;
-        fx::factor<S>(sh, s, S::ex(ip), S::ey(ip), even, odd);
-        put(std::integral_constant<int, ip>(), s, fx::equilibrium(even + odd, wr));
-        put(std::integral_constant<int, im>(), s, fx::equilibrium(even - odd, wr));
-      });
-    }
-  });
+// Pulls an FP64 node into this thread's shared memory (value i at f[i * stride]), all loads in
+// flight together and none in a register, and takes its fixed-point form and moments there; false
+// out of the range.
+template <class S, bool STREAM>
+__device__ __forceinline__ bool pull_fixed(double* f, int stride, const double* __restrict__ A,
+                                           const Geom& g, const fx::Consts& c, long long idx,
+                                           fx::State& u) {
+#pragma unroll
+  for (int i = 0; i < S::Q; ++i) {
+    const long long src = STREAM ? pull_src(g, idx, S::ex(i), S::ey(i)) : idx;
+    cp_async8(f + i * stride, A + (long long)i * g.plane + src);
+  }
+  cp_async_wait_all();
+  int low = 1 << 20;
+  const fx::Moments m = fx::gather<S>(c, f, stride, low);
+  return low >= 3 && fx::state(m, c, u);
 }
 
 // The macroscopic state of a fixed-point node in the form that the FP64 code keeps.
 __device__ __forceinline__ Macro<double> macro_of(const fx::State& u, const fx::Consts& c) {
   Macro<double> m;
-  m.rho = double(u.rho) * fx::double_of((fx::u64)(1023 - 58 + c.E) << 52);
+  m.rho = double(u.rho) * fx::pow2(c.E - 58);
   m.drho = m.rho - 1.0;
-  m.inv_rho = 0.0;   // not used by the callers
-  m.urx = u.X;
-  m.ury = u.Y;
-  m.u2 = (u.X * u.X + u.Y * u.Y) * c.inv_r2;
-  m.theta = u.th;
+  m.inv_rho = 0.0;   // this and u2 are not used by the callers
+  m.u2 = 0.0;
+  m.urx = double(u.X) * fx::pow2(-60);
+  m.ury = double(u.Y) * fx::pow2(-60);
+  m.theta = double(u.th) * fx::pow2(-60);
   return m;
 }
 
@@ -431,16 +450,16 @@ __device__ __forceinline__ Macro<double> macro_of(const fx::State& u, const fx::
 template <class S, bool STREAM>
 __device__ __forceinline__ bool bgk_fixed(const Geom& g, const fx::Consts& c,
                                           const double* __restrict__ A, double* __restrict__ B,
-                                          long long src, long long dst) {
-  fx::i64 F[S::Q];
-  if (!load_fixed<S, STREAM>(F, A, g, c, src)) return false;
+                                          long long idx, double* f, int stride) {
   fx::State u;
-  if (!fx::state(fx::moments<S>(F), c, u)) return false;
-  const fx::Site k = fx::site<S::ORDER>(u.X, u.Y, u.th, c.r2, c.inv_r2);
+  if (!pull_fixed<S, STREAM>(f, stride, A, g, c, idx, u)) return false;
+  const fx::Site k = fx::site<S::ORDER>(u, c);
   int low = 1;
-  each_equilibrium<S>(c, k, u.rho, [&](auto i, auto s, fx::i64 feq) {
-    B[(long long)i * g.plane + dst] =
-        fx::store(fx::relax(F[i], feq, c.om), fx::shell_fe<S>(s), c.E, low);
+  fx::each_equilibrium<S>(c, k, u.rho, [](const fx::ShellInfo&, int) {},
+                          [&](int h, const fx::ShellInfo& s, fx::i64 feq) {
+    const int i = s.first + h;
+    const fx::i64 F = __double_as_longlong(f[i * stride]);
+    B[(long long)i * g.plane + idx] = fx::store(fx::relax(F, feq, c.om), s.fe, c.E, low);
   });
   return low >= 1;
 }
@@ -449,14 +468,9 @@ __device__ __forceinline__ bool bgk_fixed(const Geom& g, const fx::Consts& c,
 // Block: 32 x BY threads; the x tiles start on a 32-node boundary of F.
 // (bulk_node is the per-node work, shared with the batched launch over many instances.)
 template <class S, class Real, bool DEV, bool STREAM>
-__device__ __forceinline__ void bulk_node(const Geom& g, const Consts<Real>& c,
-                                          const Real* __restrict__ A, Real* __restrict__ B,
-                                          int* flag, int x, int y) {
-  if (x < g.Fw || x >= g.Lx - g.Fe || y >= g.Ly - g.Fn) return;
-  const long long idx = gindex(g, x, y);
-  if constexpr (sizeof(Real) == 8) {
-    if (c.fx.on && bgk_fixed<S, STREAM>(g, c.fx, A, B, idx, idx)) return;
-  }
+__device__ __forceinline__ void bulk_plain(const Geom& g, const Consts<Real>& c,
+                                           const Real* __restrict__ A, Real* __restrict__ B,
+                                           int* flag, long long idx) {
   Real p[S::Q];
   load_pop<S, Real, STREAM>(p, A, g, idx);
   const Macro<Real> m = moments<S, Real, DEV>(p, c);
@@ -466,22 +480,51 @@ __device__ __forceinline__ void bulk_node(const Geom& g, const Consts<Real>& c,
   for (int i = 0; i < S::Q; ++i) B[(long long)i * g.plane + idx] = p[i];
 }
 
-// Blocks of 128 threads per SM of the FP64 interior. The fixed-point update is bound by issue and
-// by the FP64 section of its scalars, so more warps hide one behind the other until registers
-// spill. Measured at 1024^2, blocks per SM (registers): D2Q37 2 (172) 290 us, 3 (168) 237, 4 (128)
-// 215, 5 (96, spills) 264; D2Q17 4 (128) 113, 5 (96) 101; D2Q9 4 (96) 77, 8 (59) 63. FP64
-// arithmetic: 738, 385 and 203 us.
-template <class S, class Real>
-constexpr int bulk_blocks() {
-  return sizeof(Real) == 4 ? 0 : S::Q == 37 ? 4 : S::Q == 17 ? 5 : 8;   // 0: no bound
+// The FP64 arithmetic of the few nodes outside the fixed-point range, out of line: its registers
+// and code stay off the common path (here and in the frame and band kernels).
+template <class S, bool STREAM>
+__device__ __noinline__ void bulk_outside(const Geom& g, const Consts<double>& c, const double* A,
+                                          double* B, int* flag, long long idx) {
+  bulk_plain<S, double, false, STREAM>(g, c, A, B, flag, idx);
 }
 
 template <class S, class Real, bool DEV, bool STREAM>
-__global__ void __launch_bounds__(sizeof(Real) == 8 ? 128 : 256, bulk_blocks<S, Real>()) k_bulk(Geom g, Consts<Real> c, const Real* __restrict__ A,
-                                              Real* __restrict__ B, int* flag) {
+__device__ __forceinline__ void bulk_node(const Geom& g, const Consts<Real>& c,
+                                          const Real* __restrict__ A, Real* __restrict__ B,
+                                          int* flag, int x, int y, double* f, int stride) {
+  if (x < g.Fw || x >= g.Lx - g.Fe || y >= g.Ly - g.Fn) return;
+  const long long idx = gindex(g, x, y);
+  if constexpr (sizeof(Real) == 8) {
+    if (c.fx.on && bgk_fixed<S, STREAM>(g, c.fx, A, B, idx, f, stride)) return;
+    bulk_outside<S, STREAM>(g, c, A, B, flag, idx);
+  } else {
+    bulk_plain<S, Real, DEV, STREAM>(g, c, A, B, flag, idx);
+  }
+}
+
+// Blocks of 128 threads per SM of the FP64 interior. The update is bound by integer issue (about
+// 4500 instructions per D2Q37 node), so more warps help little. Measured at 1024^2, blocks per SM:
+// D2Q37 3 236 us (before the out-of-line FP64 form), 4 202, 5 199 (all its shared memory allows);
+// D2Q17 5 120, 6 95, 8 95, 10 97; D2Q9 8 53, 10 54. In FP64 arithmetic 738, 385 and 203 us.
+template <class S, class Real>
+constexpr int bulk_blocks() {
+  return sizeof(Real) == 4 ? 0 : S::Q == 37 ? 5 : S::Q == 17 ? 6 : 8;   // 0: no bound
+}
+// Shared memory of an FP64 block of n threads: one value per direction and thread.
+template <class S, class Real>
+__host__ __device__ constexpr int node_smem(int n) {
+  return sizeof(Real) == 8 ? S::Q * n : 1;
+}
+
+template <class S, class Real, bool DEV, bool STREAM>
+__global__ void __launch_bounds__(sizeof(Real) == 8 ? 128 : 256, bulk_blocks<S, Real>()) k_bulk(
+    const __grid_constant__ Geom g, const __grid_constant__ Consts<Real> c,
+    const Real* __restrict__ A, Real* __restrict__ B, int* flag) {
+  __shared__ double f[node_smem<S, Real>(128)];
   const int x0 = (g.Fw / 32) * 32;
   bulk_node<S, Real, DEV, STREAM>(g, c, A, B, flag, x0 + blockIdx.x * 32 + threadIdx.x,
-                                  g.Fs + blockIdx.y * blockDim.y + threadIdx.y);
+                                  g.Fs + blockIdx.y * blockDim.y + threadIdx.y,
+                                  f + threadIdx.y * 32 + threadIdx.x, 128);
 }
 
 // Writes the time-level moments of a node in the outer two layers of F into every edge slot
@@ -533,36 +576,91 @@ __device__ inline bool outermost(const Geom& g, int x, int y) {
   return x == 0 || x == g.Lx - 1 || (!g.py && (y == 0 || y == g.Ly - 1));
 }
 
-// 4-byte asynchronous global -> shared copy (cp.async) and the wait for all of this thread's
-// copies.
-__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
-  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.wait_all;\n" ::: "memory");
-}
-
 // Frame, phase 1: BGK plus, on P and its inner ring, the trapezoidal accumulator
 // S = Q + f_hat / 2 (Eq. PMLQ: Q^n = S^(n-1) + f_hat^n / 2, S^n = S^(n-1) + f_hat^n), and on P
 // the local part -((sigma_x + sigma_y) f_hat + sigma_x sigma_y Q) of Eq. (pml-general)
-// (-sigma (2 f_hat + sigma Q) of Eq. PMLCOLL when sigma_x = sigma_y). With the link gradient
-// the node also stores Q^n in place of S^(n-1) (no kernel of the step reads S^(n-1) after its
-// own node's phase 1; the next step writes S^(n+1) there) and adds its own share
-// +sigma Q_i(x) of the link difference, so phase 2 gathers one value per direction.
-// STAGE (FP32 table-driven launch): S^(n-1) of the node is copied into `stage` (Q values of
-// shared memory owned by this thread) by cp.async while the populations are pulled, instead
-// of being held in registers.
+// (-sigma (2 f_hat + sigma Q) of Eq. PMLCOLL when sigma_x = sigma_y). The node also stores Q^n in
+// place of S^(n-1) (no kernel of the step reads S^(n-1) after its own node's phase 1; the next
+// step writes S^(n+1) there), so phase 2 reads one value per neighbour; with the link gradient
+// it adds its own share +sigma Q_i(x) of the link difference too.
+// `stage` is shared memory owned by this thread. FP64: its node's populations, `stride` apart
+// (fixed point). STAGE (FP32 table-driven launch): Q values of S^(n-1) of the node, copied there by
+// cp.async while the populations are pulled, instead of being held in registers.
+
+// Phase 1 of an FP64 node in fixed point; false (nothing stored) out of that range. The
+// accumulator, which grows with time, stays in FP64 (four operations per direction, against about
+// 23 with the equilibrium); it is fetched into L2 during the pull and read a shell at a time.
+template <class S, bool STREAM>
+__device__ __forceinline__ bool frame1_fixed(const Geom& g, const Consts<double>& c,
+                                             const double* __restrict__ A, double* __restrict__ B,
+                                             double* __restrict__ Sold, double* __restrict__ Snew,
+                                             double* Uedge, int save_edges, double* Sedge,
+                                             int src_mask, int fi, int x, int y, double* f,
+                                             int stride) {
+  const long long idx = gindex(g, x, y);
+  const PmlLayers<double> pn = pml_layers(g, c, x, y);
+  if (pn.has_q) {
+#pragma unroll
+    for (int i = 0; i < S::Q; ++i)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(Sold + (long long)i * g.Sp + fi));
+  }
+  fx::State u;
+  if (!pull_fixed<S, STREAM>(f, stride, A, g, c.fx, idx, u)) return false;
+  if (save_edges && dist_out(g, x, y) < 2)
+    save_edge_moments(g, Uedge, x, y, macro_of(u, c.fx), c.r);
+  const double ssum = pn.sx + pn.sy, sprod = pn.sx * pn.sy;
+  const fx::Site k = fx::site<S::ORDER>(u, c.fx);
+  const bool src = src_mask && outermost(g, x, y);
+  double smom[4] = {0.0, 0.0, 0.0, 0.0};
+  double so[8];
+  fx::each_equilibrium<S>(c.fx, k, u.rho, [&](const fx::ShellInfo& s, auto size) {
+    if (pn.has_q) {
+#pragma unroll
+      for (int h = 0; h < size; ++h) so[h] = Sold[(long long)(s.first + h) * g.Sp + fi];
+    }
+  }, [&](auto h, const fx::ShellInfo& s, fx::i64 feq) {
+    const int i = s.first + h;
+    const fx::i64 F = __double_as_longlong(f[i * stride]);
+    double out = fx::store(fx::relax(F, feq, c.fx.om), s.fe, c.fx.E);
+    if (pn.has_q) {
+      const double fhat = fx::store(feq - c.fx.eqbar[i], s.fe, c.fx.E);
+      const double s0 = so[h], q = fma(0.5, fhat, s0);
+      Snew[(long long)i * g.Sp + fi] = s0 + fhat;
+      Sold[(long long)i * g.Sp + fi] = q;
+      if (pn.in_p) {
+        // link mode: with the node's own share +sigma Q_i(x) of -sigma (Q_i(x + e_i) - Q_i(x))
+        out = fma(-ssum, fhat, out);
+        out = fma(g.link && s.a ? pn.sx - sprod : -sprod, q, out);
+        if (src) {
+          const double part = -(((src_mask & 2) ? ssum * fhat : 0.0) +
+                                ((src_mask & 4) ? sprod * q : 0.0));
+          int ex, ey;
+          fx::velocity(s, h, ex, ey);
+          smom[0] += part;
+          smom[1] += ex * part;
+          smom[2] += ey * part;
+          smom[3] += (ex * ex + ey * ey) * part;
+        }
+      }
+    }
+    B[(long long)i * g.plane + idx] = out;
+  });
+  if (src) {
+    smom[1] *= c.r;
+    smom[2] *= c.r;
+    smom[3] *= 0.5 * c.r2;
+    put_pml_source(g, Sedge, x, y, smom, false);
+  }
+  return true;
+}
+
 template <class S, class Real, bool DEV, bool STREAM, bool STAGE = false>
-__device__ __forceinline__ void frame1_node(const Geom& g, const Consts<Real>& c,
-                                            const Real* __restrict__ A, Real* __restrict__ B,
-                                            Real* __restrict__ Sold,
-                                            Real* __restrict__ Snew, double* Uedge,
-                                            int save_edges, int* flag, double* Sedge,
-                                            int src_mask, int fi, Real* stage = nullptr) {
-  if (fi >= g.frame_n) return;
-  int x, y;
-  frame_xy(g, fi, x, y);
+__device__ __forceinline__ void frame1_plain(const Geom& g, const Consts<Real>& c,
+                                             const Real* __restrict__ A, Real* __restrict__ B,
+                                             Real* __restrict__ Sold,
+                                             Real* __restrict__ Snew, double* Uedge,
+                                             int save_edges, int* flag, double* Sedge,
+                                             int src_mask, int fi, int x, int y, Real* stage) {
   const int d = dist_out(g, x, y);
   const long long idx = gindex(g, x, y);
   if constexpr (STAGE) {
@@ -604,7 +702,7 @@ __device__ __forceinline__ void frame1_node(const Geom& g, const Consts<Real>& c
       const Real s0 = STAGE ? stage[i] : (kHoist ? so[i] : Sold[(long long)i * g.Sp + fi]);
       const Real q = s0 + Real(0.5) * fhat;
       Snew[(long long)i * g.Sp + fi] = s0 + fhat;
-      if (g.link) Sold[(long long)i * g.Sp + fi] = q;   // Q^n over S^(n-1), gathered by phase 2
+      Sold[(long long)i * g.Sp + fi] = q;   // Q^n over S^(n-1), read by phase 2
       Real out = p[i] + c.omega * (eq - p[i]);
       if (in_p) {
         out = out - (ssum * fhat + sprod * q);
@@ -635,32 +733,72 @@ __device__ __forceinline__ void frame1_node(const Geom& g, const Consts<Real>& c
   }
 }
 
-template <class S, class Real, bool DEV, bool STREAM>
-__global__ void __launch_bounds__(128) k_frame1(Geom g, Consts<Real> c, const Real* __restrict__ A,
-                                                Real* __restrict__ B, Real* __restrict__ Sold,
-                                                Real* __restrict__ Snew, double* Uedge, int save_edges,
-                                                int* flag, double* Sedge, int src_mask) {
-  frame1_node<S, Real, DEV, STREAM>(g, c, A, B, Sold, Snew, Uedge, save_edges, flag, Sedge,
-                                    src_mask, blockIdx.x * blockDim.x + threadIdx.x);
+template <class S, bool STREAM>
+__device__ __noinline__ void frame1_outside(const Geom& g, const Consts<double>& c, const double* A,
+                                            double* B, double* Sold, double* Snew, double* Uedge,
+                                            int save_edges, int* flag, double* Sedge, int src_mask,
+                                            int fi, int x, int y) {
+  frame1_plain<S, double, false, STREAM>(g, c, A, B, Sold, Snew, Uedge, save_edges, flag, Sedge,
+                                         src_mask, fi, x, y, nullptr);
 }
 
-// Frame, phase 2 (PML nodes): subtract sigma_y c_ix dQ_i/dx + sigma_x c_iy dQ_i/dy (sigma
-// e_i . grad Q_i when sigma_x = sigma_y) with Q = (S^(n-1) + S^n) / 2,
-// Eq. (FD-dx-center) per axis, Eq. (FD-dx-bw) along the outward normal at the outermost layer;
-// with the link gradient, the neighbour's share of the link difference (Q^n read in place).
-template <class S, class Real, bool STAGE = false>
-__device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c,
-                                            Real* __restrict__ B, const Real* __restrict__ Sold,
-                                            const Real* __restrict__ Snew, double* Sedge,
-                                            int src_mask, int fi, Real* stq = nullptr,
-                                            Real* stb = nullptr) {
+template <class S, class Real, bool DEV, bool STREAM, bool STAGE = false>
+__device__ __forceinline__ void frame1_node(const Geom& g, const Consts<Real>& c,
+                                            const Real* __restrict__ A, Real* __restrict__ B,
+                                            Real* __restrict__ Sold,
+                                            Real* __restrict__ Snew, double* Uedge,
+                                            int save_edges, int* flag, double* Sedge,
+                                            int src_mask, int fi, Real* stage = nullptr,
+                                            int stride = 0) {
   if (fi >= g.frame_n) return;
   int x, y;
   frame_xy(g, fi, x, y);
-  const PmlNode<Real> pn = pml_node<Real>(g, x, y);
+  if constexpr (sizeof(Real) == 8) {
+    if (c.fx.on && frame1_fixed<S, STREAM>(g, c, A, B, Sold, Snew, Uedge, save_edges, Sedge,
+                                           src_mask, fi, x, y, stage, stride))
+      return;
+    frame1_outside<S, STREAM>(g, c, A, B, Sold, Snew, Uedge, save_edges, flag, Sedge, src_mask, fi,
+                              x, y);
+  } else {
+    frame1_plain<S, Real, DEV, STREAM, STAGE>(g, c, A, B, Sold, Snew, Uedge, save_edges, flag,
+                                              Sedge, src_mask, fi, x, y, stage);
+  }
+}
+
+// Blocks of 128 threads per SM of the FP64 frame and band kernels. Measured on the 1024^2 frame,
+// phase 1: D2Q37 3 116 us, 4 107, 5 (spills) 124; in FP64 arithmetic 275 us.
+template <class S, class Real>
+constexpr int edge_blocks() {
+  return sizeof(Real) == 4 ? 0 : S::Q == 37 ? 4 : S::Q == 17 ? 5 : 8;
+}
+
+template <class S, class Real, bool DEV, bool STREAM>
+__global__ void __launch_bounds__(128, edge_blocks<S, Real>()) k_frame1(
+    const __grid_constant__ Geom g, const __grid_constant__ Consts<Real> c,
+                                                const Real* __restrict__ A, Real* __restrict__ B, Real* __restrict__ Sold,
+                                                Real* __restrict__ Snew, double* Uedge, int save_edges,
+                                                int* flag, double* Sedge, int src_mask) {
+  __shared__ double f[node_smem<S, Real>(128)];
+  frame1_node<S, Real, DEV, STREAM>(g, c, A, B, Sold, Snew, Uedge, save_edges, flag, Sedge,
+                                    src_mask, blockIdx.x * blockDim.x + threadIdx.x,
+                                    reinterpret_cast<Real*>(f) + threadIdx.x, 128);
+}
+
+// Frame, phase 2 (PML nodes): subtract sigma_y c_ix dQ_i/dx + sigma_x c_iy dQ_i/dy (sigma
+// e_i . grad Q_i when sigma_x = sigma_y) with Q^n as phase 1 left it in the S^(n-1) slots,
+// Eq. (FD-dx-center) per axis, Eq. (FD-dx-bw) along the outward normal at the outermost layer;
+// with the link gradient, the neighbour's share of the link difference.
+template <class S, class Real, bool STAGE = false>
+__device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c,
+                                            Real* __restrict__ B, const Real* __restrict__ Sold,
+                                            double* Sedge, int src_mask, int fi,
+                                            Real* stq = nullptr, Real* stb = nullptr) {
+  if (fi >= g.frame_n) return;
+  int x, y;
+  frame_xy(g, fi, x, y);
+  const PmlLayers<Real> pn = pml_layers(g, c, x, y);
   if (!pn.in_p) return;
-  Real sx, sy;
-  pml_sigmas(c, pn, sx, sy);
+  const Real sx = pn.sx, sy = pn.sy;
   if (g.link) {
     // link mode: the remaining -sigma Q_i(x + e_i) of -sigma (Q_i(x + e_i) - Q_i(x)), the
     // integral of sigma c_i . grad Q_i along the link the population travels (sigma_x =
@@ -722,64 +860,91 @@ __device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c
     }
     return;
   }
-  // x axis: neighbours / one-sided stencil
-  int ax0, ax1, ax2;  // frame indices; derivative = cx0*Q(ax0) + cx1*Q(ax1) + cx2*Q(ax2)
-  Real cx0, cx1, cx2;
-  if (x == 0) {  // outward normal -x: dQ/dx = -(3Q(x) - 4Q(x+1) + Q(x+2))/2
-    ax0 = fi; ax1 = frame_index(g, 1, y); ax2 = frame_index(g, 2, y);
-    cx0 = Real(-1.5); cx1 = Real(2); cx2 = Real(-0.5);
-  } else if (x == g.Lx - 1) {
-    ax0 = fi; ax1 = frame_index(g, x - 1, y); ax2 = frame_index(g, x - 2, y);
-    cx0 = Real(1.5); cx1 = Real(-2); cx2 = Real(0.5);
-  } else {
-    ax0 = frame_index(g, x + 1, y); ax1 = frame_index(g, x - 1, y); ax2 = fi;
-    cx0 = Real(0.5); cx1 = Real(-0.5); cx2 = Real(0);
-  }
-  int ay0, ay1, ay2;
-  Real cy0, cy1, cy2;
-  if (g.py) {  // periodic y: central difference with wrap
-    ay0 = frame_index(g, x, y + 1 < g.Ly ? y + 1 : 0);
-    ay1 = frame_index(g, x, y > 0 ? y - 1 : g.Ly - 1);
-    ay2 = fi;
-    cy0 = Real(0.5); cy1 = Real(-0.5); cy2 = Real(0);
-  } else if (y == 0) {
-    ay0 = fi; ay1 = frame_index(g, x, 1); ay2 = frame_index(g, x, 2);
-    cy0 = Real(-1.5); cy1 = Real(2); cy2 = Real(-0.5);
-  } else if (y == g.Ly - 1) {
-    ay0 = fi; ay1 = frame_index(g, x, y - 1); ay2 = frame_index(g, x, y - 2);
-    cy0 = Real(1.5); cy1 = Real(-2); cy2 = Real(0.5);
-  } else {
-    ay0 = frame_index(g, x, y + 1); ay1 = frame_index(g, x, y - 1); ay2 = fi;
-    cy0 = Real(0.5); cy1 = Real(-0.5); cy2 = Real(0);
-  }
   const long long idx = gindex(g, x, y);
   const bool src = (src_mask & 1) && outermost(g, x, y);   // Appendix term I
-  double smom[4] = {0.0, 0.0, 0.0, 0.0};   // FP64 sums (cancellation)
+  // offsets and coefficients of the per-axis differences: sigma_y c_x dQ/dx is e_x times
+  // cx[0] Q(ax[0]) + cx[1] Q(ax[1]) + cx[2] Q(x), the last only at an outermost layer
+  int ax0 = x + 1, ax1 = x - 1, ay0 = y + 1, ay1 = y - 1;
+  Real cx0 = Real(0.5) * sy, cx1 = -cx0, cx2 = Real(0);
+  Real cy0 = Real(0.5) * sx, cy1 = -cy0, cy2 = Real(0);
+  if (x == 0) {   // outward normal -x: dQ/dx = -(3 Q(x) - 4 Q(x+1) + Q(x+2)) / 2
+    ax1 = 2;
+    cx0 = Real(2) * sy; cx1 = Real(-0.5) * sy; cx2 = Real(-1.5) * sy;
+  } else if (x == g.Lx - 1) {
+    ax0 = x - 1; ax1 = x - 2;
+    cx0 = Real(-2) * sy; cx1 = Real(0.5) * sy; cx2 = Real(1.5) * sy;
+  }
+  if (g.py) {     // periodic y: central difference with wrap
+    if (ay0 == g.Ly) ay0 = 0;
+    if (ay1 < 0) ay1 = g.Ly - 1;
+  } else if (y == 0) {
+    ay1 = 2;
+    cy0 = Real(2) * sx; cy1 = Real(-0.5) * sx; cy2 = Real(-1.5) * sx;
+  } else if (y == g.Ly - 1) {
+    ay0 = y - 1; ay1 = y - 2;
+    cy0 = Real(-2) * sx; cy1 = Real(0.5) * sx; cy2 = Real(1.5) * sx;
+  }
+  const int fx0 = frame_index(g, ax0, y), fx1 = frame_index(g, ax1, y);
+  const int fy0 = frame_index(g, x, ay0), fy1 = frame_index(g, x, ay1);
+  const bool xe = x == 0 || x == g.Lx - 1, ye = !g.py && (y == 0 || y == g.Ly - 1);
+  // G directions' loads in flight together: a store to B holds back every later load of B. One at
+  // a time the 1024^2 FP64 frame takes 121 us against 102, and an outermost layer's warps, which
+  // also run the one-sided form, make a 64^2 grid's phase 2 take 37 us against 23.
+  if (!xe && !ye) {
+    constexpr int G = 6;
 #pragma unroll
-  for (int i = 0; i < S::Q; ++i) {
-    const Real* so = Sold + (long long)i * g.Sp;
-    const Real* sn = Snew + (long long)i * g.Sp;
-    Real gq = 0;   // sigma_y c_x dQ/dx + sigma_x c_y dQ/dy, with 2Q
-    if (S::ex(i) != 0) {
-      const Real dx = cx0 * (__ldg(so + ax0) + __ldg(sn + ax0)) +
-                      cx1 * (__ldg(so + ax1) + __ldg(sn + ax1)) +
-                      cx2 * (__ldg(so + ax2) + __ldg(sn + ax2));
-      gq += sy * Real(S::ex(i)) * dx;
+    for (int i0 = 1; i0 < S::Q; i0 += G) {
+      Real v[G], q[G][4];
+#pragma unroll
+      for (int h = 0; h < G; ++h) {
+        const int i = i0 + h;
+        if (i >= S::Q) continue;
+        const Real* s = Sold + (long long)i * g.Sp;
+        v[h] = B[(long long)i * g.plane + idx];
+        if (S::ex(i) != 0) { q[h][0] = __ldg(s + fx0); q[h][1] = __ldg(s + fx1); }
+        if (S::ey(i) != 0) { q[h][2] = __ldg(s + fy0); q[h][3] = __ldg(s + fy1); }
+      }
+#pragma unroll
+      for (int h = 0; h < G; ++h) {
+        const int i = i0 + h;
+        if (i >= S::Q) continue;
+        if (S::ex(i) != 0) v[h] -= (Real(S::ex(i)) * cx0) * (q[h][0] - q[h][1]);
+        if (S::ey(i) != 0) v[h] -= (Real(S::ey(i)) * cy0) * (q[h][2] - q[h][3]);
+        B[(long long)i * g.plane + idx] = v[h];
+      }
     }
-    if (S::ey(i) != 0) {
-      const Real dy = cy0 * (__ldg(so + ay0) + __ldg(sn + ay0)) +
-                      cy1 * (__ldg(so + ay1) + __ldg(sn + ay1)) +
-                      cy2 * (__ldg(so + ay2) + __ldg(sn + ay2));
-      gq += sx * Real(S::ey(i)) * dy;
+    return;
+  }
+  double smom[4] = {0.0, 0.0, 0.0, 0.0};   // FP64 sums (cancellation)
+  constexpr int G = 4;
+#pragma unroll
+  for (int i0 = 1; i0 < S::Q; i0 += G) {
+    Real v[G], q[G][5];
+#pragma unroll
+    for (int h = 0; h < G; ++h) {
+      const int i = i0 + h;
+      if (i >= S::Q) continue;
+      const Real* s = Sold + (long long)i * g.Sp;
+      v[h] = B[(long long)i * g.plane + idx];
+      if (S::ex(i) != 0) { q[h][0] = __ldg(s + fx0); q[h][1] = __ldg(s + fx1); }
+      if (S::ey(i) != 0) { q[h][2] = __ldg(s + fy0); q[h][3] = __ldg(s + fy1); }
+      q[h][4] = __ldg(s + fi);
     }
-    Real* b = B + (long long)i * g.plane + idx;
-    *b = *b - Real(0.5) * gq;   // Q = (S^(n-1) + S^n) / 2
-    if (src) {
-      const double part = -0.5 * double(gq);
-      smom[0] += part;
-      smom[1] += double(S::ex(i)) * part;
-      smom[2] += double(S::ey(i)) * part;
-      smom[3] += double(S::ex(i) * S::ex(i) + S::ey(i) * S::ey(i)) * part;
+#pragma unroll
+    for (int h = 0; h < G; ++h) {
+      const int i = i0 + h;
+      if (i >= S::Q) continue;
+      Real gq = 0;   // sigma_y c_x dQ/dx + sigma_x c_y dQ/dy
+      if (S::ex(i) != 0) gq += Real(S::ex(i)) * (cx0 * q[h][0] + cx1 * q[h][1] + cx2 * q[h][4]);
+      if (S::ey(i) != 0) gq += Real(S::ey(i)) * (cy0 * q[h][2] + cy1 * q[h][3] + cy2 * q[h][4]);
+      B[(long long)i * g.plane + idx] = v[h] - gq;
+      if (src) {
+        const double part = -double(gq);
+        smom[0] += part;
+        smom[1] += double(S::ex(i)) * part;
+        smom[2] += double(S::ey(i)) * part;
+        smom[3] += double(S::ex(i) * S::ex(i) + S::ey(i) * S::ey(i)) * part;
+      }
     }
   }
   if (src) {
@@ -792,10 +957,9 @@ __device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c
 
 template <class S, class Real>
 __global__ void __launch_bounds__(128) k_frame2(Geom g, Consts<Real> c, Real* __restrict__ B,
-                                                const Real* __restrict__ Sold,
-                                                const Real* __restrict__ Snew, double* Sedge,
+                                                const Real* __restrict__ Sold, double* Sedge,
                                                 int src_mask) {
-  frame2_node<S, Real>(g, c, B, Sold, Snew, Sedge, src_mask, blockIdx.x * blockDim.x + threadIdx.x);
+  frame2_node<S, Real>(g, c, B, Sold, Sedge, src_mask, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 __device__ inline void gamma_xy(const Geom& g, int t, int& x, int& y) {
@@ -834,39 +998,73 @@ __device__ inline int q_slot(const Geom& g, int x, int y) {
 // Link mode with a PML (Sold != nullptr): the node also advances its accumulator
 // S^n = S^(n-1) + f_hat^n (slot frame_n + t) from the moments of its pre-collision state, and
 // stores Q^n = S^(n-1) + f_hat^n / 2 in place of S^(n-1) for the frame's phase 2.
-template <class S, class Real, bool DEV, bool STREAM>
-__device__ __forceinline__ void gamma_node(const Geom& g, const Consts<Real>& c,
-                                           const BcParams& bc, const Real* __restrict__ A,
-                                           Real* __restrict__ B,
-                                           const double* __restrict__ Vtgt,
-                                           Real* __restrict__ Sold,
-                                           Real* __restrict__ Snew, int t) {
-  if (t >= g.ngamma) return;
-  int x, y;
-  gamma_xy(g, t, x, y);
-  // rows beyond a periodic y axis are copied from the finished rows they image (k_wrap_y)
-  if (g.py && (y < 0 || y >= g.Ly)) return;
-  const long long dst = gindex(g, x, y);
-  int sx, sy;
-  if (bc.bc == 0) {
-    sx = (x + g.Lx) % g.Lx;
-    sy = (y + g.Ly) % g.Ly;
-  } else {
-    sx = min(max(x, 0), g.Lx - 1);
-    sy = min(max(y, 0), g.Ly - 1);
+// The same for an FP64 node in fixed point; false (nothing stored) where the fluid node or the
+// target is out of its range.
+template <class S, bool STREAM>
+__device__ __forceinline__ bool gamma_fixed(const Geom& g, const Consts<double>& c,
+                                            const BcParams& bc, const double* __restrict__ A,
+                                            double* __restrict__ B,
+                                            const double* __restrict__ Vtgt, int b,
+                                            double* __restrict__ Sold,
+                                            double* __restrict__ Snew, int t, long long src,
+                                            long long dst, double* f, int stride) {
+  fx::State u;
+  if (!pull_fixed<S, STREAM>(f, stride, A, g, c.fx, src, u)) return false;
+  fx::Site k = fx::site<S::ORDER>(u, c.fx);
+  if (b >= 0) {
+    const double X = bc.r * Vtgt[g.nb + b], Y = bc.r * Vtgt[2 * g.nb + b];
+    const double rho = Vtgt[b] * fx::pow2(-c.fx.E), th = Vtgt[3 * g.nb + b] - 1.0;
+    if (!(rho < 2.0 && rho > 0.5 && fabs(X) < 2.0 && fabs(Y) < 2.0 && fabs(th) < 2.0)) return false;
+    fx::State ut;
+    ut.rho = fx::fixed60(rho) >> 2;
+    ut.X = fx::fixed60(X);
+    ut.Y = fx::fixed60(Y);
+    ut.th = fx::fixed60(th);
+    if (!fx::in_range(ut)) return false;
+    // (1 - omega) f_neq(x_f) in place of f, then the targets' equilibrium
+    fx::each_equilibrium<S>(c.fx, k, u.rho, [](const fx::ShellInfo&, int) {},
+                            [&](int h, const fx::ShellInfo& s, fx::i64 feq) {
+      double* at = f + (s.first + h) * stride;
+      const fx::i64 F = __double_as_longlong(*at);
+      *at = __longlong_as_double(fx::relax(F, feq, c.fx.om) - feq);
+    });
+    k = fx::site<S::ORDER>(ut, c.fx);
+    u.rho = ut.rho;
   }
+  double so[8];
+  fx::each_equilibrium<S>(c.fx, k, u.rho, [&](const fx::ShellInfo& s, auto size) {
+    if (Sold) {
+#pragma unroll
+      for (int h = 0; h < size; ++h)
+        so[h] = Sold[(long long)(s.first + h) * g.Sp + g.frame_n + t];
+    }
+  }, [&](auto h, const fx::ShellInfo& s, fx::i64 feq) {
+    const int i = s.first + h;
+    const fx::i64 F = __double_as_longlong(f[i * stride]);
+    B[(long long)i * g.plane + dst] =
+        fx::store(b >= 0 ? F + feq : fx::relax(F, feq, c.fx.om), s.fe, c.fx.E);
+    if (Sold) {
+      const long long n = (long long)i * g.Sp + g.frame_n + t;
+      const double fh = fx::store(feq - c.fx.eqbar[i], s.fe, c.fx.E), s0 = so[h];
+      Snew[n] = s0 + fh;
+      Sold[n] = fma(0.5, fh, s0);   // Q^n in place, gathered by the frame's phase 2
+    }
+  });
+  return true;
+}
+
+template <class S, class Real, bool DEV, bool STREAM>
+__device__ __forceinline__ void gamma_plain(const Geom& g, const Consts<Real>& c,
+                                            const BcParams& bc, const Real* __restrict__ A,
+                                            Real* __restrict__ B,
+                                            const double* __restrict__ Vtgt, int b,
+                                            Real* __restrict__ Sold,
+                                            Real* __restrict__ Snew, int t, long long src,
+                                            long long dst) {
   Real p[S::Q];
-  load_pop<S, Real, STREAM>(p, A, g, gindex(g, sx, sy));
+  load_pop<S, Real, STREAM>(p, A, g, src);
   const Macro<Real> m = moments<S, Real, DEV>(p, c);
-  const bool xo = x < 0 || x >= g.Lx, yo = y < 0 || y >= g.Ly;
-  if (bc.bc == 2 && xo != yo) {
-    // edge band node: index into the target arrays
-    int b;
-    const int M = g.M, Lx = g.Lx, Ly = g.Ly;
-    if (x < 0) b = (-x - 1) * Ly + y;
-    else if (x >= Lx) b = M * Ly + (x - Lx) * Ly + y;
-    else if (y < 0) b = 2 * M * Ly + (-y - 1) * Lx + x;
-    else b = 2 * M * Ly + M * Lx + (y - Ly) * Lx + x;
+  if (b >= 0) {
     Macro<Real> mt;
     const double trho = Vtgt[b], tux = Vtgt[g.nb + b], tuy = Vtgt[2 * g.nb + b],
                  tT = Vtgt[3 * g.nb + b];
@@ -923,14 +1121,65 @@ __device__ __forceinline__ void gamma_node(const Geom& g, const Consts<Real>& c,
   for (int i = 0; i < S::Q; ++i) B[(long long)i * g.plane + dst] = p[i];
 }
 
+template <class S, bool STREAM>
+__device__ __noinline__ void gamma_outside(const Geom& g, const Consts<double>& c,
+                                           const BcParams& bc, const double* A, double* B,
+                                           const double* Vtgt, int b, double* Sold, double* Snew,
+                                           int t, long long src, long long dst) {
+  gamma_plain<S, double, false, STREAM>(g, c, bc, A, B, Vtgt, b, Sold, Snew, t, src, dst);
+}
+
 template <class S, class Real, bool DEV, bool STREAM>
-__global__ void __launch_bounds__(128) k_gamma(Geom g, Consts<Real> c, BcParams bc,
-                                               const Real* __restrict__ A, Real* __restrict__ B,
+__device__ __forceinline__ void gamma_node(const Geom& g, const Consts<Real>& c,
+                                           const BcParams& bc, const Real* __restrict__ A,
+                                           Real* __restrict__ B,
+                                           const double* __restrict__ Vtgt,
+                                           Real* __restrict__ Sold,
+                                           Real* __restrict__ Snew, int t, double* f,
+                                           int stride) {
+  if (t >= g.ngamma) return;
+  int x, y;
+  gamma_xy(g, t, x, y);
+  // rows beyond a periodic y axis are copied from the finished rows they image (k_wrap_y)
+  if (g.py && (y < 0 || y >= g.Ly)) return;
+  const long long dst = gindex(g, x, y);
+  int sx, sy;
+  if (bc.bc == 0) {
+    sx = (x + g.Lx) % g.Lx;
+    sy = (y + g.Ly) % g.Ly;
+  } else {
+    sx = min(max(x, 0), g.Lx - 1);
+    sy = min(max(y, 0), g.Ly - 1);
+  }
+  const bool xo = x < 0 || x >= g.Lx, yo = y < 0 || y >= g.Ly;
+  int b = -1;   // edge band node: index into the target arrays
+  if (bc.bc == 2 && xo != yo) {
+    const int M = g.M, Lx = g.Lx, Ly = g.Ly;
+    if (x < 0) b = (-x - 1) * Ly + y;
+    else if (x >= Lx) b = M * Ly + (x - Lx) * Ly + y;
+    else if (y < 0) b = 2 * M * Ly + (-y - 1) * Lx + x;
+    else b = 2 * M * Ly + M * Lx + (y - Ly) * Lx + x;
+  }
+  const long long src = gindex(g, sx, sy);
+  if constexpr (sizeof(Real) == 8) {
+    if (c.fx.on && gamma_fixed<S, STREAM>(g, c, bc, A, B, Vtgt, b, Sold, Snew, t, src, dst, f, stride))
+      return;
+    gamma_outside<S, STREAM>(g, c, bc, A, B, Vtgt, b, Sold, Snew, t, src, dst);
+  } else {
+    gamma_plain<S, Real, DEV, STREAM>(g, c, bc, A, B, Vtgt, b, Sold, Snew, t, src, dst);
+  }
+}
+
+template <class S, class Real, bool DEV, bool STREAM>
+__global__ void __launch_bounds__(128, edge_blocks<S, Real>()) k_gamma(
+    const __grid_constant__ Geom g, const __grid_constant__ Consts<Real> c,
+    const __grid_constant__ BcParams bc, const Real* __restrict__ A, Real* __restrict__ B,
                                                const double* __restrict__ Vtgt,
                                                Real* __restrict__ Sold,
                                                Real* __restrict__ Snew) {
+  __shared__ double f[node_smem<S, Real>(128)];
   gamma_node<S, Real, DEV, STREAM>(g, c, bc, A, B, Vtgt, Sold, Snew,
-                                   blockIdx.x * blockDim.x + threadIdx.x);
+                                   blockIdx.x * blockDim.x + threadIdx.x, f + threadIdx.x, 128);
 }
 
 // Periodic y axis: the M rows below y = 0 and above y = Ly - 1 (boundary columns included)

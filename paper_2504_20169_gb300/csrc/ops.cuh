@@ -222,15 +222,18 @@ struct MemberDev {
 };
 
 template <class S, class Real, bool DEV>
-__global__ void __launch_bounds__(256, (bulk_blocks<S, Real>() + 1) / 2) kb_bulk(const MemberDev<Real>* __restrict__ mem,
+__global__ void __launch_bounds__(256, bulk_blocks<S, Real>() / 2) kb_bulk(const MemberDev<Real>* __restrict__ mem,
                                                const int* __restrict__ tab) {
+  extern __shared__ double bsh[];   // FP64: the nodes of the block (node_smem values)
   const int* e = tab + 3 * blockIdx.x;
   const MemberDev<Real>& md = mem[e[0]];
   const Geom g = md.g;
   const int x0 = (g.Fw / 32) * 32;
   bulk_node<S, Real, DEV, true>(g, md.c, md.A, md.B, md.flag,
                                 x0 + e[1] * blockDim.x + threadIdx.x,
-                                g.Fs + e[2] * blockDim.y + threadIdx.y);
+                                g.Fs + e[2] * blockDim.y + threadIdx.y,
+                                bsh + threadIdx.y * blockDim.x + threadIdx.x,
+                                blockDim.x * blockDim.y);
 }
 
 template <class S>
@@ -244,7 +247,7 @@ __global__ void __launch_bounds__(256) kb_pml_fused(const MemberDev<float>* __re
 }
 
 template <class S, class Real, bool DEV>
-__global__ void __launch_bounds__(128) kb_frame1(const MemberDev<Real>* __restrict__ mem,
+__global__ void __launch_bounds__(128, edge_blocks<S, Real>()) kb_frame1(const MemberDev<Real>* __restrict__ mem,
                                                  const int* __restrict__ tab) {
   const int* e = tab + 2 * blockIdx.x;
   const MemberDev<Real>& md = mem[e[0]];
@@ -257,9 +260,10 @@ __global__ void __launch_bounds__(128) kb_frame1(const MemberDev<Real>* __restri
                                           md.src_mask, e[1] * blockDim.x + threadIdx.x,
                                           reinterpret_cast<Real*>(stage) + threadIdx.x * S::Q);
   } else {
+    __shared__ double f[node_smem<S, Real>(128)];
     frame1_node<S, Real, DEV, true>(g, md.c, md.A, md.B, md.Sold, md.Snew, md.Uedge_out,
                                     md.bc.bc == 2 ? 1 : 0, md.flag, md.Sedge_out, md.src_mask,
-                                    e[1] * blockDim.x + threadIdx.x);
+                                    e[1] * blockDim.x + threadIdx.x, f + threadIdx.x, 128);
   }
 }
 
@@ -272,26 +276,27 @@ __global__ void __launch_bounds__(128) kb_frame2(const MemberDev<Real>* __restri
   if constexpr (sizeof(Real) == 4) {
     // FP32: the gathers and the loads of B are staged in shared memory by cp.async
     __shared__ float stq[128 * S::Q], stb[128 * S::Q];
-    frame2_node<S, Real, true>(g, md.c, md.B, md.Sold, md.Snew, md.Sedge_out, md.src_mask,
+    frame2_node<S, Real, true>(g, md.c, md.B, md.Sold, md.Sedge_out, md.src_mask,
                                e[1] * blockDim.x + threadIdx.x,
                                reinterpret_cast<Real*>(stq) + threadIdx.x * S::Q,
                                reinterpret_cast<Real*>(stb) + threadIdx.x * S::Q);
   } else {
-    frame2_node<S, Real>(g, md.c, md.B, md.Sold, md.Snew, md.Sedge_out, md.src_mask,
+    frame2_node<S, Real>(g, md.c, md.B, md.Sold, md.Sedge_out, md.src_mask,
                          e[1] * blockDim.x + threadIdx.x);
   }
 }
 
 template <class S, class Real, bool DEV>
-__global__ void __launch_bounds__(128) kb_gamma(const MemberDev<Real>* __restrict__ mem,
+__global__ void __launch_bounds__(128, edge_blocks<S, Real>()) kb_gamma(const MemberDev<Real>* __restrict__ mem,
                                                 const int* __restrict__ tab) {
   const int* e = tab + 2 * blockIdx.x;
   const MemberDev<Real>& md = mem[e[0]];
   const Geom g = md.g;
   const bool link = g.link && has_pml(g);
+  __shared__ double f[node_smem<S, Real>(128)];
   gamma_node<S, Real, DEV, true>(g, md.c, md.bc, md.A, md.B, md.Vtgt,
                                  link ? md.Sold : nullptr, link ? md.Snew : nullptr,
-                                 e[1] * blockDim.x + threadIdx.x);
+                                 e[1] * blockDim.x + threadIdx.x, f + threadIdx.x, 128);
 }
 
 template <class Real>
@@ -394,8 +399,7 @@ struct Ops {
       mark(6, fs);
       if (has_pml(g) && !fused)
         k_frame2<S, Real><<<(g.frame_n + 127) / 128, 128, 0, fs>>>(
-            g, c, B, static_cast<const Real*>(d.Sold), static_cast<const Real*>(d.Snew),
-            d.Sedge_out, src_mask);
+            g, c, B, static_cast<const Real*>(d.Sold), d.Sedge_out, src_mask);
       mark(7, fs);
       if (!link) band();
     }
@@ -491,6 +495,9 @@ struct Ops {
         if (dev >= 0 && dev < 64) done[dev] = true;
       }
     }
+    if constexpr (!DEV)
+      return cudaFuncSetAttribute(kb_bulk<S, Real, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(double) * node_smem<S, Real>(256));
     if constexpr (DEV) {
       cudaError_t e = cudaFuncSetAttribute(k_pml_fused<S, true>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
@@ -645,7 +652,8 @@ struct Ops {
     if (p.n_f2) kb_frame2<S, Real><<<p.n_f2, 128, 0, fs>>>(mem, p.f2_tab);
     // the interiors of every member on st
     if (p.n_bulk)
-      kb_bulk<S, Real, DEV><<<p.n_bulk, dim3(p.tx, p.by), 0, st>>>(mem, p.bulk_tab);
+      kb_bulk<S, Real, DEV><<<p.n_bulk, dim3(p.tx, p.by),
+                              sizeof(double) * node_smem<S, Real>(p.tx * p.by), st>>>(mem, p.bulk_tab);
     if (aux) {
       cudaEventRecord(join, aux);
       cudaStreamWaitEvent(st, join, 0);

@@ -53,30 +53,18 @@ static void collide(T* f, T omega) {
 }
 template <class S>
 static bool collide_fixed(double* p, const fx::Consts& c) {
-  fx::i64 F[S::Q];
+  double f[37];
+  std::memcpy(f, p, sizeof f);
   int low = 1 << 20, out = 1;
-  for (int s = 0; s < S::NSHELL; ++s)
-    for (int i = S::shell_first(s); i < S::shell_first(s) + S::shell_size(s); ++i)
-      F[i] = fx::load(p[i], fx::shell_fe<S>(s), c.E, low);
+  const fx::Moments m = fx::gather<S>(c, f, 1, low);
   fx::State u;
-  if (low < 3 || !fx::state(fx::moments<S>(F), c, u)) return false;
-  const fx::Site k = fx::site<S::ORDER>(u.X, u.Y, u.th, c.r2, c.inv_r2);
-  for (int s = 0; s < S::NSHELL; ++s) {
-    const fx::Limbs wr = fx::shell_weight<S>(c, s, u.rho);
-    const int i0 = S::shell_first(s), n = S::shell_size(s), fe = fx::shell_fe<S>(s);
-    if (n == 1) {
-      p[i0] = fx::store(fx::relax(F[i0], fx::equilibrium(k.A0, wr), c.om), fe, c.E, out);
-      continue;
-    }
-    const fx::Shell sh = fx::shell<S>(fx::shell_far<S>(s) ? fx::coarse<S::ORDER>(k) : k, s);
-    for (int h = 0; h < n / 2; ++h) {
-      fx::i64 even, odd;
-      const int ip = i0 + h, im = ip + n / 2;
-      fx::factor<S>(sh, s, S::ex(ip), S::ey(ip), even, odd);
-      p[ip] = fx::store(fx::relax(F[ip], fx::equilibrium(even + odd, wr), c.om), fe, c.E, out);
-      p[im] = fx::store(fx::relax(F[im], fx::equilibrium(even - odd, wr), c.om), fe, c.E, out);
-    }
-  }
+  if (low < 3 || !fx::state(m, c, u)) return false;
+  const fx::Site k = fx::site<S::ORDER>(u, c);
+  fx::each_equilibrium<S>(c, k, u.rho, [](const fx::ShellInfo&, int) {},
+                          [&](int h, const fx::ShellInfo& s, fx::i64 feq) {
+    const fx::i64 F = (fx::i64)fx::bits_of(f[s.first + h]);
+    p[s.first + h] = fx::store(fx::relax(F, feq, c.om), s.fe, c.E, out);
+  });
   return out >= 1;
 }
 template <class S>
@@ -84,11 +72,12 @@ static void run(double umax, double tmax, double rlo, double rhi, double noise, 
   fx::Consts c;
   std::memset(&c, 0, sizeof c);
   c.E = (int)std::lround(std::log2(0.5 * (rlo + rhi)));
-  c.r2 = (double)(R * R);
-  c.inv_r2 = 1.0 / c.r2;
-  c.om = fx::split((fx::i64)std::llrint(std::ldexp((ld)omega, 61)));
-  for (int s = 0; s < S::NSHELL; ++s)
-    c.w[s] = fx::split((fx::i64)std::llrint(std::ldexp(W[S::shell_first(s)], fx::shell_k<S>(s) + 62)));
+  c.r2 = fx::split((fx::i64)std::llrint(std::ldexp(R * R, 60)));
+  c.inv_r2 = fx::split((fx::i64)std::llrint(std::ldexp(1 / (R * R), 60)));
+  c.om = fx::factor((fx::i64)std::llrint(std::ldexp((ld)omega, 61)));
+  double w[37];
+  for (int i = 0; i < S::Q; ++i) w[i] = (double)W[i];
+  if (!fx::make_shells<S>(w, c.shell)) std::exit(3);
   std::mt19937_64 gen(7);
   auto U = [&]() { return std::ldexp((double)(gen() >> 11), -52) - 1.0; };
   const int N = 20000;
