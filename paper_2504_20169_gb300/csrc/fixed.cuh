@@ -138,12 +138,6 @@ LBM_HD i64 prod(Limbs a, Limbs b) {
   return (i64)((u64)((i64)a.h * b.h) << up) + (m >> (32 - up));
 }
 
-// A shell as the loops see it: velocities of base (a, b), a >= b, from direction `first` on.
-struct ShellInfo {
-  int first, a, b, fe;
-  Factor w;          // weight w 2^k in units of 2^-62
-};
-
 // Kinds of shell: (0, 0), then (a, 0), then (a, a), then (a, b).
 template <class S>
 LBM_HD constexpr int kind_of(int s) {
@@ -155,6 +149,30 @@ LBM_HD constexpr int kind_count(int kind) {
   for (int s = 0; s < S::NSHELL; ++s) n += kind_of<S>(s) == kind ? 1 : 0;
   return n;
 }
+
+// Position of a direction's shell in the order of kinds.
+template <class S>
+LBM_HD constexpr int shell_position(int i) {
+  int at = 0, mine = 0;
+  for (int s = 0; s < S::NSHELL; ++s)
+    if (i >= S::shell_first(s)) mine = s;
+  for (int s = 0; s < S::NSHELL; ++s)
+    if (kind_of<S>(s) < kind_of<S>(mine) || (kind_of<S>(s) == kind_of<S>(mine) && s < mine)) ++at;
+  return at;
+}
+// The shells of one of four warps that share 32 nodes: at most 12 of 37 directions, 5 of 17, 4 of 9.
+template <class S>
+LBM_HD unsigned warp_shells(int w) {
+  if (S::Q == 37) return w == 0 ? 0x40u : w == 1 ? 0x80u : w == 2 ? 0x07u : 0x38u;
+  if (S::Q == 17) return w == 0 ? 0x02u : w == 1 ? 0x04u : w == 2 ? 0x08u : 0x11u;
+  return w == 0 ? 0x02u : w == 1 ? 0x04u : w == 2 ? 0x01u : 0x00u;
+}
+
+// A shell as the loops see it: velocities of base (a, b), a >= b, from direction `first` on.
+struct ShellInfo {
+  int first, a, b, fe;
+  Factor w;          // weight w 2^k in units of 2^-62
+};
 
 // f 2^(fe - E) of a double f >= 0. `low` takes the smallest right shift seen: below 3 a
 // population is out of range (2^59 units or more, negative, infinite or NaN).
@@ -289,10 +307,14 @@ LBM_HD Factor shell_weight(const ShellInfo& h, i64 rho58) { return factor(2 * mu
 // F + omega (feq - F); |feq - F| < 2^60.
 LBM_HD i64 relax(i64 F, i64 feq, Factor om) { return F + mul((feq - F) * 8, om); }
 
+constexpr unsigned kAllShells = 0xffu;
+
 // put(h, shell, feq) for every direction shell.first + h with its equilibrium in fixed point;
-// pre(shell, size) before a shell (h and size are integral constants).
+// pre(shell, size) before a shell (h and size are integral constants). Only the shells in `mask`
+// (bit k: c.shell[k]).
 template <class S, class Pre, class Put>
-LBM_HD void each_equilibrium(const Consts& c, const Site& k, i64 rho58, Pre pre, Put put) {
+LBM_HD void each_equilibrium(const Consts& c, const Site& k, i64 rho58, Pre pre, Put put,
+                             unsigned mask = kAllShells) {
   constexpr int axis = kind_count<S>(1), diag = kind_count<S>(2), octet = kind_count<S>(3);
   using std::integral_constant;
   integral_constant<int, 0> h0;
@@ -304,13 +326,14 @@ LBM_HD void each_equilibrium(const Consts& c, const Site& k, i64 rho58, Pre pre,
   integral_constant<int, 6> h6;
   integral_constant<int, 7> h7;
   integral_constant<int, 8> h8;
-  {
+  if (mask & 1u) {
     const ShellInfo& h = c.shell[0];
     pre(h, h1);
     put(h0, h, mul(k.A0, shell_weight(h, rho58)));
   }
 #pragma unroll 1
   for (int j = 0; j < axis; ++j) {
+    if (!(mask >> (1 + j) & 1u)) continue;
     const ShellInfo& h = c.shell[1 + j];
     pre(h, h4);
     const Factor w = shell_weight(h, rho58);
@@ -334,6 +357,7 @@ LBM_HD void each_equilibrium(const Consts& c, const Site& k, i64 rho58, Pre pre,
   }
 #pragma unroll 1
   for (int j = 0; j < diag; ++j) {
+    if (!(mask >> (1 + axis + j) & 1u)) continue;
     const ShellInfo& h = c.shell[1 + axis + j];
     pre(h, h4);
     const Factor w = shell_weight(h, rho58);
@@ -358,6 +382,7 @@ LBM_HD void each_equilibrium(const Consts& c, const Site& k, i64 rho58, Pre pre,
   }
 #pragma unroll 1
   for (int j = 0; j < octet; ++j) {
+    if (!(mask >> (1 + axis + diag + j) & 1u)) continue;
     const ShellInfo& h = c.shell[1 + axis + diag + j];
     pre(h, h8);
     const Factor w = shell_weight(h, rho58);
@@ -410,10 +435,11 @@ struct Moments {
   i64 rho, jx, jy, e2;
 };
 
-// Reads a node's doubles at f[i * stride], leaves their integers there and sums them; `low` as in
-// load().
+// Reads a node's doubles at f[i * stride], leaves their integers there and sums them (the shells in
+// `mask`); `low` as in load().
 template <class S>
-LBM_HD Moments gather(const Consts& c, double* f, int stride, int& low) {
+LBM_HD Moments gather(const Consts& c, double* f, int stride, int& low,
+                      unsigned mask = kAllShells) {
   constexpr int axis = kind_count<S>(1), diag = kind_count<S>(2), octet = kind_count<S>(3);
   auto get = [&](const ShellInfo& s, int h) {
     double* at = f + (s.first + h) * stride;
@@ -431,24 +457,27 @@ LBM_HD Moments gather(const Consts& c, double* f, int stride, int& low) {
     m.jy += (y + half) >> sh;
     m.e2 += n * sum;
   };
-  {
+  if (mask & 1u) {
     const ShellInfo& s = c.shell[0];
     m.rho = get(s, 0) << (58 - s.fe);   // the rest weight is above 1/8: fe = 56 or 57
   }
 #pragma unroll 1
   for (int j = 0; j < axis; ++j) {
+    if (!(mask >> (1 + j) & 1u)) continue;
     const ShellInfo& s = c.shell[1 + j];
     const i64 p0 = get(s, 0), p1 = get(s, 1), p2 = get(s, 2), p3 = get(s, 3);
     add(s, s.a * s.a, p0 + p1 + p2 + p3, s.a * (p0 - p2), s.a * (p1 - p3));
   }
 #pragma unroll 1
   for (int j = 0; j < diag; ++j) {
+    if (!(mask >> (1 + axis + j) & 1u)) continue;
     const ShellInfo& s = c.shell[1 + axis + j];
     const i64 p0 = get(s, 0), p1 = get(s, 1), p2 = get(s, 2), p3 = get(s, 3);
     add(s, 2 * s.a * s.a, p0 + p1 + p2 + p3, s.a * (p0 - p1 - p2 + p3), s.a * (p0 + p1 - p2 - p3));
   }
 #pragma unroll 1
   for (int j = 0; j < octet; ++j) {
+    if (!(mask >> (1 + axis + diag + j) & 1u)) continue;
     const ShellInfo& s = c.shell[1 + axis + diag + j];
     const i64 p0 = get(s, 0), p1 = get(s, 1), p2 = get(s, 2), p3 = get(s, 3);
     const i64 p4 = get(s, 4), p5 = get(s, 5), p6 = get(s, 6), p7 = get(s, 7);

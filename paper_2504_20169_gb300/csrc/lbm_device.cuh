@@ -428,6 +428,49 @@ __device__ __forceinline__ bool pull_fixed(double* f, int stride, const double* 
   return low >= 3 && fx::state(m, c, u);
 }
 
+// Four warps on 32 nodes: on a small grid a kernel's time is the latency of one warp's chain (about
+// 7000 instructions for a frame node on D2Q37), so each warp takes a part of the shells. All
+// threads of the block call pull_split (live: the lane has a node); every warp ends with the
+// node's whole state. The values are those of pull_fixed.
+struct SplitShared {
+  fx::i64 part[4][4][32];
+  int low[4][32];
+};
+template <class S, bool STREAM>
+__device__ __forceinline__ bool pull_split(double* f, SplitShared& sh, int warp, int lane, bool live,
+                                           const double* __restrict__ A, const Geom& g,
+                                           const fx::Consts& c, long long idx, fx::State& u) {
+  const unsigned mask = fx::warp_shells<S>(warp);
+  fx::Moments m{0, 0, 0, 0};
+  int low = 1 << 20;
+  if (live) {
+#pragma unroll
+    for (int i = 0; i < S::Q; ++i) {
+      const long long src = STREAM ? pull_src(g, idx, S::ex(i), S::ey(i)) : idx;
+      if (mask >> fx::shell_position<S>(i) & 1u)
+        cp_async8(f + i * 32 + lane, A + (long long)i * g.plane + src);
+    }
+    cp_async_wait_all();
+    m = fx::gather<S>(c, f + lane, 32, low, mask);
+  }
+  sh.part[warp][0][lane] = m.rho;
+  sh.part[warp][1][lane] = m.jx;
+  sh.part[warp][2][lane] = m.jy;
+  sh.part[warp][3][lane] = m.e2;
+  sh.low[warp][lane] = low;
+  __syncthreads();
+  fx::Moments t{0, 0, 0, 0};
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    t.rho += sh.part[w][0][lane];
+    t.jx += sh.part[w][1][lane];
+    t.jy += sh.part[w][2][lane];
+    t.e2 += sh.part[w][3][lane];
+    low = min(low, sh.low[w][lane]);
+  }
+  return live && low >= 3 && fx::state(t, c, u);
+}
+
 // The macroscopic state of a fixed-point node in the form that the FP64 code keeps.
 __device__ __forceinline__ Macro<double> macro_of(const fx::State& u, const fx::Consts& c) {
   Macro<double> m;
@@ -587,27 +630,18 @@ __device__ inline bool outermost(const Geom& g, int x, int y) {
 // (fixed point). STAGE (FP32 table-driven launch): Q values of S^(n-1) of the node, copied there by
 // cp.async while the populations are pulled, instead of being held in registers.
 
-// Phase 1 of an FP64 node in fixed point; false (nothing stored) out of that range. The
-// accumulator, which grows with time, stays in FP64 (four operations per direction, against about
-// 23 with the equilibrium); it is fetched into L2 during the pull and read a shell at a time.
-template <class S, bool STREAM>
-__device__ __forceinline__ bool frame1_fixed(const Geom& g, const Consts<double>& c,
-                                             const double* __restrict__ A, double* __restrict__ B,
-                                             double* __restrict__ Sold, double* __restrict__ Snew,
-                                             double* Uedge, int save_edges, double* Sedge,
-                                             int src_mask, int fi, int x, int y, double* f,
-                                             int stride) {
+// Phase 1 of an FP64 node in fixed point from its state u and its integers at f[i * stride]: the
+// shells in `mask`. The accumulator, which grows with time, stays in FP64 (four operations per
+// direction, against about 23 with the equilibrium); it is fetched into L2 during the pull and
+// read a shell at a time.
+template <class S>
+__device__ __forceinline__ void frame1_put(const Geom& g, const Consts<double>& c,
+                                           double* __restrict__ B, double* __restrict__ Sold,
+                                           double* __restrict__ Snew, double* Sedge, int src_mask,
+                                           int fi, int x, int y, const PmlLayers<double>& pn,
+                                           const fx::State& u, const double* f, int stride,
+                                           unsigned mask) {
   const long long idx = gindex(g, x, y);
-  const PmlLayers<double> pn = pml_layers(g, c, x, y);
-  if (pn.has_q) {
-#pragma unroll
-    for (int i = 0; i < S::Q; ++i)
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(Sold + (long long)i * g.Sp + fi));
-  }
-  fx::State u;
-  if (!pull_fixed<S, STREAM>(f, stride, A, g, c.fx, idx, u)) return false;
-  if (save_edges && dist_out(g, x, y) < 2)
-    save_edge_moments(g, Uedge, x, y, macro_of(u, c.fx), c.r);
   const double ssum = pn.sx + pn.sy, sprod = pn.sx * pn.sy;
   const fx::Site k = fx::site<S::ORDER>(u, c.fx);
   const bool src = src_mask && outermost(g, x, y);
@@ -644,13 +678,34 @@ __device__ __forceinline__ bool frame1_fixed(const Geom& g, const Consts<double>
       }
     }
     B[(long long)i * g.plane + idx] = out;
-  });
+  }, mask);
   if (src) {
     smom[1] *= c.r;
     smom[2] *= c.r;
     smom[3] *= 0.5 * c.r2;
     put_pml_source(g, Sedge, x, y, smom, false);
   }
+}
+
+// Phase 1 of an FP64 node; false (nothing stored) out of the fixed-point range.
+template <class S, bool STREAM>
+__device__ __forceinline__ bool frame1_fixed(const Geom& g, const Consts<double>& c,
+                                             const double* __restrict__ A, double* __restrict__ B,
+                                             double* __restrict__ Sold, double* __restrict__ Snew,
+                                             double* Uedge, int save_edges, double* Sedge,
+                                             int src_mask, int fi, int x, int y, double* f,
+                                             int stride) {
+  const PmlLayers<double> pn = pml_layers(g, c, x, y);
+  if (pn.has_q) {
+#pragma unroll
+    for (int i = 0; i < S::Q; ++i)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(Sold + (long long)i * g.Sp + fi));
+  }
+  fx::State u;
+  if (!pull_fixed<S, STREAM>(f, stride, A, g, c.fx, gindex(g, x, y), u)) return false;
+  if (save_edges && dist_out(g, x, y) < 2)
+    save_edge_moments(g, Uedge, x, y, macro_of(u, c.fx), c.r);
+  frame1_put<S>(g, c, B, Sold, Snew, Sedge, src_mask, fi, x, y, pn, u, f, stride, fx::kAllShells);
   return true;
 }
 
@@ -765,6 +820,35 @@ __device__ __forceinline__ void frame1_node(const Geom& g, const Consts<Real>& c
   }
 }
 
+// Phase 1 with four warps on 32 nodes (all threads of the block call it; no PML source terms).
+template <class S>
+__device__ __forceinline__ void frame1_split(const Geom& g, const Consts<double>& c,
+                                             const double* __restrict__ A, double* __restrict__ B,
+                                             double* __restrict__ Sold, double* __restrict__ Snew,
+                                             double* Uedge, int save_edges, int* flag, int fi,
+                                             int warp, int lane, double* f, SplitShared& sh) {
+  const bool live = fi < g.frame_n;
+  int x = 0, y = 0;
+  if (live) frame_xy(g, fi, x, y);
+  const PmlLayers<double> pn = pml_layers(g, c, x, y);
+  const unsigned mask = fx::warp_shells<S>(warp);
+  if (live && pn.has_q) {
+#pragma unroll
+    for (int i = 0; i < S::Q; ++i)
+      if (mask >> fx::shell_position<S>(i) & 1u)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(Sold + (long long)i * g.Sp + fi));
+  }
+  fx::State u;
+  const bool ok = pull_split<S, true>(f, sh, warp, lane, live, A, g, c.fx, gindex(g, x, y), u);
+  if (ok) {
+    if (warp == 0 && save_edges && dist_out(g, x, y) < 2)
+      save_edge_moments(g, Uedge, x, y, macro_of(u, c.fx), c.r);
+    frame1_put<S>(g, c, B, Sold, Snew, nullptr, 0, fi, x, y, pn, u, f + lane, 32, mask);
+  } else if (live && warp == 0) {
+    frame1_outside<S, true>(g, c, A, B, Sold, Snew, Uedge, save_edges, flag, nullptr, 0, fi, x, y);
+  }
+}
+
 // Blocks of 128 threads per SM of the FP64 frame and band kernels. Measured on the 1024^2 frame,
 // phase 1: D2Q37 3 116 us, 4 107, 5 (spills) 124; in FP64 arithmetic 275 us.
 template <class S, class Real>
@@ -788,11 +872,12 @@ __global__ void __launch_bounds__(128, edge_blocks<S, Real>()) k_frame1(
 // e_i . grad Q_i when sigma_x = sigma_y) with Q^n as phase 1 left it in the S^(n-1) slots,
 // Eq. (FD-dx-center) per axis, Eq. (FD-dx-bw) along the outward normal at the outermost layer;
 // with the link gradient, the neighbour's share of the link difference.
-template <class S, class Real, bool STAGE = false>
+template <class S, class Real, bool STAGE = false, int FIRST = 1, int LAST = S::Q>
 __device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c,
                                             Real* __restrict__ B, const Real* __restrict__ Sold,
                                             double* Sedge, int src_mask, int fi,
                                             Real* stq = nullptr, Real* stb = nullptr) {
+  // FIRST .. LAST - 1: the directions that this call takes (all, or a warp's share)
   if (fi >= g.frame_n) return;
   int x, y;
   frame_xy(g, fi, x, y);
@@ -825,8 +910,7 @@ __device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c
     constexpr bool kHoistB = sizeof(Real) == 4 && !STAGE;
     Real qg[S::Q], bg[S::Q];
 #pragma unroll
-    for (int i = 0; i < S::Q; ++i) {
-      if (S::ex(i) == 0 && S::ey(i) == 0) continue;
+    for (int i = FIRST; i < LAST; ++i) {
       const int nb = rl ? fi + S::ey(i) * rl + S::ex(i) : q_slot(g, x + S::ex(i), y + S::ey(i));
       if constexpr (STAGE) {
         cp_async4(stq + i, Sold + (long long)i * g.Sp + nb);
@@ -838,8 +922,7 @@ __device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c
     }
     if constexpr (STAGE) cp_async_wait_all();
 #pragma unroll
-    for (int i = 0; i < S::Q; ++i) {
-      if (S::ex(i) == 0 && S::ey(i) == 0) continue;
+    for (int i = FIRST; i < LAST; ++i) {
       const Real* sq = Sold + (long long)i * g.Sp;
       const Real qn = STAGE ? stq[i] : qg[i];
       Real* b = B + (long long)i * g.plane + idx;
@@ -893,12 +976,12 @@ __device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c
   if (!xe && !ye) {
     constexpr int G = 6;
 #pragma unroll
-    for (int i0 = 1; i0 < S::Q; i0 += G) {
+    for (int i0 = FIRST; i0 < LAST; i0 += G) {
       Real v[G], q[G][4];
 #pragma unroll
       for (int h = 0; h < G; ++h) {
         const int i = i0 + h;
-        if (i >= S::Q) continue;
+        if (i >= LAST) continue;
         const Real* s = Sold + (long long)i * g.Sp;
         v[h] = B[(long long)i * g.plane + idx];
         if (S::ex(i) != 0) { q[h][0] = __ldg(s + fx0); q[h][1] = __ldg(s + fx1); }
@@ -907,7 +990,7 @@ __device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c
 #pragma unroll
       for (int h = 0; h < G; ++h) {
         const int i = i0 + h;
-        if (i >= S::Q) continue;
+        if (i >= LAST) continue;
         if (S::ex(i) != 0) v[h] -= (Real(S::ex(i)) * cx0) * (q[h][0] - q[h][1]);
         if (S::ey(i) != 0) v[h] -= (Real(S::ey(i)) * cy0) * (q[h][2] - q[h][3]);
         B[(long long)i * g.plane + idx] = v[h];
@@ -918,12 +1001,12 @@ __device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c
   double smom[4] = {0.0, 0.0, 0.0, 0.0};   // FP64 sums (cancellation)
   constexpr int G = 4;
 #pragma unroll
-  for (int i0 = 1; i0 < S::Q; i0 += G) {
+  for (int i0 = FIRST; i0 < LAST; i0 += G) {
     Real v[G], q[G][5];
 #pragma unroll
     for (int h = 0; h < G; ++h) {
       const int i = i0 + h;
-      if (i >= S::Q) continue;
+      if (i >= LAST) continue;
       const Real* s = Sold + (long long)i * g.Sp;
       v[h] = B[(long long)i * g.plane + idx];
       if (S::ex(i) != 0) { q[h][0] = __ldg(s + fx0); q[h][1] = __ldg(s + fx1); }
@@ -933,7 +1016,7 @@ __device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c
 #pragma unroll
     for (int h = 0; h < G; ++h) {
       const int i = i0 + h;
-      if (i >= S::Q) continue;
+      if (i >= LAST) continue;
       Real gq = 0;   // sigma_y c_x dQ/dx + sigma_x c_y dQ/dy
       if (S::ex(i) != 0) gq += Real(S::ex(i)) * (cx0 * q[h][0] + cx1 * q[h][1] + cx2 * q[h][4]);
       if (S::ey(i) != 0) gq += Real(S::ey(i)) * (cy0 * q[h][2] + cy1 * q[h][3] + cy2 * q[h][4]);
@@ -998,36 +1081,37 @@ __device__ inline int q_slot(const Geom& g, int x, int y) {
 // Link mode with a PML (Sold != nullptr): the node also advances its accumulator
 // S^n = S^(n-1) + f_hat^n (slot frame_n + t) from the moments of its pre-collision state, and
 // stores Q^n = S^(n-1) + f_hat^n / 2 in place of S^(n-1) for the frame's phase 2.
-// The same for an FP64 node in fixed point; false (nothing stored) where the fluid node or the
-// target is out of its range.
-template <class S, bool STREAM>
-__device__ __forceinline__ bool gamma_fixed(const Geom& g, const Consts<double>& c,
-                                            const BcParams& bc, const double* __restrict__ A,
-                                            double* __restrict__ B,
-                                            const double* __restrict__ Vtgt, int b,
-                                            double* __restrict__ Sold,
-                                            double* __restrict__ Snew, int t, long long src,
-                                            long long dst, double* f, int stride) {
-  fx::State u;
-  if (!pull_fixed<S, STREAM>(f, stride, A, g, c.fx, src, u)) return false;
+// The target state of band node b in fixed point; false out of its range.
+__device__ __forceinline__ bool target_state(const Geom& g, const fx::Consts& c, const BcParams& bc,
+                                             const double* __restrict__ Vtgt, int b,
+                                             fx::State& ut) {
+  const double X = bc.r * Vtgt[g.nb + b], Y = bc.r * Vtgt[2 * g.nb + b];
+  const double rho = Vtgt[b] * fx::pow2(-c.E), th = Vtgt[3 * g.nb + b] - 1.0;
+  if (!(rho < 2.0 && rho > 0.5 && fabs(X) < 2.0 && fabs(Y) < 2.0 && fabs(th) < 2.0)) return false;
+  ut.rho = fx::fixed60(rho) >> 2;
+  ut.X = fx::fixed60(X);
+  ut.Y = fx::fixed60(Y);
+  ut.th = fx::fixed60(th);
+  return fx::in_range(ut);
+}
+
+// The same for an FP64 node in fixed point from the fluid node's state u and integers and, on an
+// edge band (b >= 0), the target state ut: the shells in `mask`.
+template <class S>
+__device__ __forceinline__ void gamma_put(const Geom& g, const Consts<double>& c,
+                                          double* __restrict__ B, int b,
+                                          double* __restrict__ Sold, double* __restrict__ Snew,
+                                          int t, long long dst, fx::State u, const fx::State& ut,
+                                          double* f, int stride, unsigned mask) {
   fx::Site k = fx::site<S::ORDER>(u, c.fx);
   if (b >= 0) {
-    const double X = bc.r * Vtgt[g.nb + b], Y = bc.r * Vtgt[2 * g.nb + b];
-    const double rho = Vtgt[b] * fx::pow2(-c.fx.E), th = Vtgt[3 * g.nb + b] - 1.0;
-    if (!(rho < 2.0 && rho > 0.5 && fabs(X) < 2.0 && fabs(Y) < 2.0 && fabs(th) < 2.0)) return false;
-    fx::State ut;
-    ut.rho = fx::fixed60(rho) >> 2;
-    ut.X = fx::fixed60(X);
-    ut.Y = fx::fixed60(Y);
-    ut.th = fx::fixed60(th);
-    if (!fx::in_range(ut)) return false;
     // (1 - omega) f_neq(x_f) in place of f, then the targets' equilibrium
     fx::each_equilibrium<S>(c.fx, k, u.rho, [](const fx::ShellInfo&, int) {},
                             [&](int h, const fx::ShellInfo& s, fx::i64 feq) {
       double* at = f + (s.first + h) * stride;
       const fx::i64 F = __double_as_longlong(*at);
       *at = __longlong_as_double(fx::relax(F, feq, c.fx.om) - feq);
-    });
+    }, mask);
     k = fx::site<S::ORDER>(ut, c.fx);
     u.rho = ut.rho;
   }
@@ -1049,8 +1133,7 @@ __device__ __forceinline__ bool gamma_fixed(const Geom& g, const Consts<double>&
       Snew[n] = s0 + fh;
       Sold[n] = fma(0.5, fh, s0);   // Q^n in place, gathered by the frame's phase 2
     }
-  });
-  return true;
+  }, mask);
 }
 
 template <class S, class Real, bool DEV, bool STREAM>
@@ -1129,6 +1212,36 @@ __device__ __noinline__ void gamma_outside(const Geom& g, const Consts<double>& 
   gamma_plain<S, double, false, STREAM>(g, c, bc, A, B, Vtgt, b, Sold, Snew, t, src, dst);
 }
 
+// Boundary node t: its place (dst), the fluid node it copies (src), its index b in the target
+// arrays (-1 off the edge bands); false if another kernel fills it (rows beyond a periodic y axis
+// are copied from the finished rows they image, k_wrap_y).
+__device__ __forceinline__ bool gamma_place(const Geom& g, const BcParams& bc, int t, long long& src,
+                                            long long& dst, int& b) {
+  int x, y;
+  gamma_xy(g, t, x, y);
+  if (g.py && (y < 0 || y >= g.Ly)) return false;
+  dst = gindex(g, x, y);
+  int sx, sy;
+  if (bc.bc == 0) {
+    sx = (x + g.Lx) % g.Lx;
+    sy = (y + g.Ly) % g.Ly;
+  } else {
+    sx = min(max(x, 0), g.Lx - 1);
+    sy = min(max(y, 0), g.Ly - 1);
+  }
+  src = gindex(g, sx, sy);
+  const bool xo = x < 0 || x >= g.Lx, yo = y < 0 || y >= g.Ly;
+  b = -1;
+  if (bc.bc == 2 && xo != yo) {
+    const int M = g.M, Lx = g.Lx, Ly = g.Ly;
+    if (x < 0) b = (-x - 1) * Ly + y;
+    else if (x >= Lx) b = M * Ly + (x - Lx) * Ly + y;
+    else if (y < 0) b = 2 * M * Ly + (-y - 1) * Lx + x;
+    else b = 2 * M * Ly + M * Lx + (y - Ly) * Lx + x;
+  }
+  return true;
+}
+
 template <class S, class Real, bool DEV, bool STREAM>
 __device__ __forceinline__ void gamma_node(const Geom& g, const Consts<Real>& c,
                                            const BcParams& bc, const Real* __restrict__ A,
@@ -1138,36 +1251,40 @@ __device__ __forceinline__ void gamma_node(const Geom& g, const Consts<Real>& c,
                                            Real* __restrict__ Snew, int t, double* f,
                                            int stride) {
   if (t >= g.ngamma) return;
-  int x, y;
-  gamma_xy(g, t, x, y);
-  // rows beyond a periodic y axis are copied from the finished rows they image (k_wrap_y)
-  if (g.py && (y < 0 || y >= g.Ly)) return;
-  const long long dst = gindex(g, x, y);
-  int sx, sy;
-  if (bc.bc == 0) {
-    sx = (x + g.Lx) % g.Lx;
-    sy = (y + g.Ly) % g.Ly;
-  } else {
-    sx = min(max(x, 0), g.Lx - 1);
-    sy = min(max(y, 0), g.Ly - 1);
-  }
-  const bool xo = x < 0 || x >= g.Lx, yo = y < 0 || y >= g.Ly;
-  int b = -1;   // edge band node: index into the target arrays
-  if (bc.bc == 2 && xo != yo) {
-    const int M = g.M, Lx = g.Lx, Ly = g.Ly;
-    if (x < 0) b = (-x - 1) * Ly + y;
-    else if (x >= Lx) b = M * Ly + (x - Lx) * Ly + y;
-    else if (y < 0) b = 2 * M * Ly + (-y - 1) * Lx + x;
-    else b = 2 * M * Ly + M * Lx + (y - Ly) * Lx + x;
-  }
-  const long long src = gindex(g, sx, sy);
+  long long src, dst;
+  int b;
+  if (!gamma_place(g, bc, t, src, dst, b)) return;
   if constexpr (sizeof(Real) == 8) {
-    if (c.fx.on && gamma_fixed<S, STREAM>(g, c, bc, A, B, Vtgt, b, Sold, Snew, t, src, dst, f, stride))
-      return;
-    gamma_outside<S, STREAM>(g, c, bc, A, B, Vtgt, b, Sold, Snew, t, src, dst);
+    fx::State u, ut;
+    if (c.fx.on && (b < 0 || target_state(g, c.fx, bc, Vtgt, b, ut)) &&
+        pull_fixed<S, STREAM>(f, stride, A, g, c.fx, src, u))
+      gamma_put<S>(g, c, B, b, Sold, Snew, t, dst, u, ut, f, stride, fx::kAllShells);
+    else
+      gamma_outside<S, STREAM>(g, c, bc, A, B, Vtgt, b, Sold, Snew, t, src, dst);
   } else {
     gamma_plain<S, Real, DEV, STREAM>(g, c, bc, A, B, Vtgt, b, Sold, Snew, t, src, dst);
   }
+}
+
+// With four warps on 32 nodes (all threads of the block call it).
+template <class S>
+__device__ __forceinline__ void gamma_split(const Geom& g, const Consts<double>& c,
+                                            const BcParams& bc, const double* __restrict__ A,
+                                            double* __restrict__ B,
+                                            const double* __restrict__ Vtgt,
+                                            double* __restrict__ Sold, double* __restrict__ Snew,
+                                            int t, int warp, int lane, double* f,
+                                            SplitShared& sh) {
+  long long src = 0, dst = 0;
+  int b = -1;
+  const bool live = t < g.ngamma && gamma_place(g, bc, t, src, dst, b);
+  fx::State u, ut;
+  const bool in = pull_split<S, true>(f, sh, warp, lane, live, A, g, c.fx, src, u);
+  const bool ok = in && (b < 0 || target_state(g, c.fx, bc, Vtgt, b, ut));
+  if (ok)
+    gamma_put<S>(g, c, B, b, Sold, Snew, t, dst, u, ut, f + lane, 32, fx::warp_shells<S>(warp));
+  else if (live && warp == 0)
+    gamma_outside<S, true>(g, c, bc, A, B, Vtgt, b, Sold, Snew, t, src, dst);
 }
 
 template <class S, class Real, bool DEV, bool STREAM>

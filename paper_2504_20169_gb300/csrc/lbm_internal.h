@@ -38,6 +38,7 @@ struct Dev {
   // PML frame on aux2 (both may be null: everything then runs in order on st).
   cudaStream_t aux, aux2;
   cudaEvent_t fork, join, join2;
+  cudaEvent_t begun;   // the blocks of the frame's first kernel have all started
   // optional timing: when ev is set, event 2k / 2k+1 are recorded around kernel class k
   // (0 characteristic targets, 1 interior, 2 frame phase 1, 3 frame phase 2, 4 boundary band)
   cudaEvent_t* ev;
@@ -78,6 +79,7 @@ struct BatchPlan {
   int tgt_threads = 0, q = 0;
   int tx = 32, by = 4;        // bulk tile shape (blockDim)
   bool link = false;
+  bool split = false;         // small launches may run four warps on 32 nodes (FP64)
   void* mem = nullptr;
 };
 
@@ -98,7 +100,7 @@ struct OpsTable {
                             int by, BatchPlan* plan);
   cudaError_t (*batch_step)(const BatchPlan& plan, int which, cudaStream_t st, cudaStream_t aux,
                             cudaStream_t aux2, cudaEvent_t fork, cudaEvent_t join,
-                            cudaEvent_t join2);
+                            cudaEvent_t join2, cudaEvent_t begun);
 };
 
 void batch_plan_free(BatchPlan* plan);

@@ -299,6 +299,48 @@ __global__ void __launch_bounds__(128, edge_blocks<S, Real>()) kb_gamma(const Me
                                  e[1] * blockDim.x + threadIdx.x, f + threadIdx.x, 128);
 }
 
+// Small FP64 launches: four warps on 32 nodes, four blocks to an entry of the table (entries whose
+// member is out of the fixed-point arithmetic altogether have one warp do the node).
+template <class S>
+__global__ void __launch_bounds__(128) kb_frame1_split(const MemberDev<double>* __restrict__ mem,
+                                                       const int* __restrict__ tab) {
+  __shared__ double f[S::Q * 32];
+  __shared__ SplitShared sh;
+  const int* e = tab + 2 * (blockIdx.x >> 2);
+  const MemberDev<double>& md = mem[e[0]];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  frame1_split<S>(md.g, md.c, md.A, md.B, md.Sold, md.Snew, md.Uedge_out, md.bc.bc == 2 ? 1 : 0,
+                  md.flag, e[1] * 128 + (blockIdx.x & 3) * 32 + lane, warp, lane, f, sh);
+}
+
+template <class S>
+__global__ void __launch_bounds__(128) kb_frame2_split(const MemberDev<double>* __restrict__ mem,
+                                                       const int* __restrict__ tab) {
+  const int* e = tab + 2 * (blockIdx.x >> 2);
+  const MemberDev<double>& md = mem[e[0]];
+  const Geom g = md.g;
+  const int warp = threadIdx.x >> 5, fi = e[1] * 128 + (blockIdx.x & 3) * 32 + (threadIdx.x & 31);
+  constexpr int n = (S::Q - 1) / 4;
+  if (warp == 0) frame2_node<S, double, false, 1, 1 + n>(g, md.c, md.B, md.Sold, nullptr, 0, fi);
+  else if (warp == 1) frame2_node<S, double, false, 1 + n, 1 + 2 * n>(g, md.c, md.B, md.Sold, nullptr, 0, fi);
+  else if (warp == 2) frame2_node<S, double, false, 1 + 2 * n, 1 + 3 * n>(g, md.c, md.B, md.Sold, nullptr, 0, fi);
+  else frame2_node<S, double, false, 1 + 3 * n, S::Q>(g, md.c, md.B, md.Sold, nullptr, 0, fi);
+}
+
+template <class S>
+__global__ void __launch_bounds__(128) kb_gamma_split(const MemberDev<double>* __restrict__ mem,
+                                                      const int* __restrict__ tab) {
+  __shared__ double f[S::Q * 32];
+  __shared__ SplitShared sh;
+  const int* e = tab + 2 * (blockIdx.x >> 2);
+  const MemberDev<double>& md = mem[e[0]];
+  const bool link = md.g.link && has_pml(md.g);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  gamma_split<S>(md.g, md.c, md.bc, md.A, md.B, md.Vtgt, link ? md.Sold : nullptr,
+                 link ? md.Snew : nullptr, e[1] * 128 + (blockIdx.x & 3) * 32 + lane, warp, lane, f,
+                 sh);
+}
+
 template <class Real>
 __global__ void __launch_bounds__(256) kb_wrap_y(const MemberDev<Real>* __restrict__ mem,
                                                  const int* __restrict__ tab) {
@@ -308,10 +350,75 @@ __global__ void __launch_bounds__(256) kb_wrap_y(const MemberDev<Real>* __restri
   wrap_y_elem<Real>(g, md.B, (long long)e[1] * blockDim.x + threadIdx.x, blockIdx.y);
 }
 
+// Largest launches (blocks of 128 nodes) that take the four-warp kernels: they shorten the chain of
+// a launch that leaves the chip idle and cost throughput (each warp forms the site's scalars) where
+// it is full. Measured, FP64, one warp / four warps on a node: 64^2 grid (20 blocks) phase 1 33 / 15
+// us, phase 2 26 / 14, band 20 / 13; 300^2 D2Q17 (209 blocks) 22.7 / 20.1, 20.2 / 18.3, 14.2 / 12.1;
+// 1024^2 (band 103 blocks) 32 / 23, (phase 1 1088 blocks) 109 / 139. The interior gains nothing at
+// any size (128^2: 12.5 / 12.6 us).
+constexpr int kSplitBlocks = 256;
+
+// Launches `kernel` on s; `begun` (may be null) is an event that fires once all its blocks have
+// started. The interior waits for that event of the frame's first kernel: the frame, on the
+// critical path and short of blocks, goes first, and the interior fills the SMs as it drains.
+// Without it a graph starts the two in either order (link gradient, 1024^2, eight steps to a
+// graph: 162 us a step against 125; 512^2 printed 54 against 46, 2048^2 286 against 271).
+template <class... P, class... A>
+inline void launch_begun(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s,
+                         cudaEvent_t begun, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at = {};
+  if (begun) {
+    at.id = cudaLaunchAttributeLaunchCompletionEvent;
+    at.val.launchCompletionEvent.event = begun;
+    at.val.launchCompletionEvent.flags = 0;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+  }
+  cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 template <class S, class Real, bool DEV>
 struct Ops {
   static const Consts<Real>& consts(const Dev& d) {
     if constexpr (sizeof(Real) == 8) return d.cd; else return d.cf;
+  }
+
+  static void launch_frame1(const BatchPlan& p, const MemberDev<Real>* m, cudaStream_t s,
+                            cudaEvent_t begun) {
+    if (!p.n_f1) return;
+    const int* tab = p.f1_tab;
+    if constexpr (!DEV) {
+      if (p.split && p.n_f1 <= kSplitBlocks) {
+        launch_begun(kb_frame1_split<S>, 4 * p.n_f1, 128, 0, s, begun, m, tab);
+        return;
+      }
+    }
+    launch_begun(kb_frame1<S, Real, DEV>, p.n_f1, 128, 0, s, begun, m, tab);
+  }
+  static void launch_frame2(const BatchPlan& p, const MemberDev<Real>* m, cudaStream_t s) {
+    if (!p.n_f2) return;
+    if constexpr (!DEV) {
+      if (p.split && p.n_f2 <= kSplitBlocks) {
+        kb_frame2_split<S><<<4 * p.n_f2, 128, 0, s>>>(m, p.f2_tab);
+        return;
+      }
+    }
+    kb_frame2<S, Real><<<p.n_f2, 128, 0, s>>>(m, p.f2_tab);
+  }
+  static void launch_band(const BatchPlan& p, const MemberDev<Real>* m, cudaStream_t s) {
+    if (!p.n_band) return;
+    if constexpr (!DEV) {
+      if (p.split && p.n_band <= kSplitBlocks) {
+        kb_gamma_split<S><<<4 * p.n_band, 128, 0, s>>>(m, p.band_tab);
+        return;
+      }
+    }
+    kb_gamma<S, Real, DEV><<<p.n_band, 128, 0, s>>>(m, p.band_tab);
   }
 
   template <bool STREAM>
@@ -324,9 +431,9 @@ struct Ops {
     // read A and write disjoint parts of B
     const bool link = g.link && has_pml(g);
     const cudaStream_t bs = d.aux ? d.aux : d.st;
-    // link mode: the gradient pass reads the boundary nodes' new accumulator, so the frame
-    // runs on the boundary stream in the order frame phase 1, band, frame phase 2
-    const cudaStream_t fs = link ? bs : (d.aux2 ? d.aux2 : bs);
+    // link mode: the gradient pass reads the boundary nodes' new accumulator, so phase 2 of the
+    // frame waits for the band
+    const cudaStream_t fs = d.aux2 ? d.aux2 : bs;
     auto mark = [&](int k, cudaStream_t s) {
       if (d.ev) cudaEventRecord(d.ev[k], s);
     };
@@ -352,21 +459,31 @@ struct Ops {
     mark(1, bs);
     mark(4, fs);
     if (pl) {
+      const cudaEvent_t begun = d.aux ? d.begun : nullptr;
       if constexpr (DEV) {
-        if (pl->n_frame)
-          kb_pml_fused<S><<<pl->n_frame, 256, pl->frame_smem, fs>>>(
-              reinterpret_cast<const MemberDev<float>*>(pm), pl->frame_tab);
+        if (pl->n_frame) {
+          const int* tab = pl->frame_tab;
+          launch_begun(kb_pml_fused<S>, pl->n_frame, 256, pl->frame_smem, fs, begun,
+                       reinterpret_cast<const MemberDev<float>*>(pm), tab);
+        }
       }
-      if (pl->n_f1) kb_frame1<S, Real, DEV><<<pl->n_f1, 128, 0, fs>>>(pm, pl->f1_tab);
+      launch_frame1(*pl, pm, fs, begun);
+      if (begun) cudaStreamWaitEvent(d.st, begun, 0);
       mark(5, fs);
       auto band_b = [&]() {
         mark(8, bs);
-        if (pl->n_band) kb_gamma<S, Real, DEV><<<pl->n_band, 128, 0, bs>>>(pm, pl->band_tab);
+        launch_band(*pl, pm, bs);
         mark(9, bs);
       };
-      if (link) band_b();
+      if (link) {
+        band_b();
+        if (fs != bs) {
+          cudaEventRecord(d.join, bs);
+          cudaStreamWaitEvent(fs, d.join, 0);
+        }
+      }
       mark(6, fs);
-      if (pl->n_f2) kb_frame2<S, Real><<<pl->n_f2, 128, 0, fs>>>(pm, pl->f2_tab);
+      launch_frame2(*pl, pm, fs);
       mark(7, fs);
       if (!link) band_b();
     }
@@ -395,7 +512,13 @@ struct Ops {
       mark(9, bs);
     };
     if (!pl) {
-      if (link) band();
+      if (link) {
+        band();
+        if (fs != bs) {
+          cudaEventRecord(d.join, bs);
+          cudaStreamWaitEvent(fs, d.join, 0);
+        }
+      }
       mark(6, fs);
       if (has_pml(g) && !fused)
         k_frame2<S, Real><<<(g.frame_n + 127) / 128, 128, 0, fs>>>(
@@ -542,6 +665,10 @@ struct Ops {
     p.by = by;
     p.q = S::Q;
     p.link = n > 0 && dev0[0]->g.link;
+    // the four-warp kernels: FP64 members in fixed point, without PML source terms
+    p.split = !DEV;
+    for (int m = 0; m < n; ++m)
+      if (!dev0[m]->cd.fx.on || dev0[m]->bc.pml_source & 7) p.split = false;
     std::vector<int> bulk, frame, f1, f2, band, tgt, wrap;
     for (int m = 0; m < n; ++m) {
       const Geom& g = dev0[m]->g;
@@ -625,10 +752,10 @@ struct Ops {
 
   static cudaError_t batch_step(const BatchPlan& p, int which, cudaStream_t st, cudaStream_t aux,
                                 cudaStream_t aux2, cudaEvent_t fork, cudaEvent_t join,
-                                cudaEvent_t join2) {
+                                cudaEvent_t join2, cudaEvent_t begun) {
     const MemberDev<Real>* mem = static_cast<const MemberDev<Real>*>(p.desc[which]);
     const cudaStream_t bs = aux ? aux : st;
-    const cudaStream_t fs = p.link ? bs : (aux2 ? aux2 : bs);
+    const cudaStream_t fs = aux2 ? aux2 : bs;
     if (aux) {
       cudaEventRecord(fork, st);
       cudaStreamWaitEvent(aux, fork, 0);
@@ -638,18 +765,26 @@ struct Ops {
     cudaError_t e = launch_nrbc_batch(p.tgt[which], p.tgt_tab, p.n_tgt, sizeof(Real) == 4,
                                       p.tgt_threads, p.tgt_smem, bs);
     if (e != cudaSuccess) return e;
-    auto band = [&]() {
-      if (p.n_band) kb_gamma<S, Real, DEV><<<p.n_band, 128, 0, bs>>>(mem, p.band_tab);
-    };
+    auto band = [&]() { launch_band(p, mem, bs); };
     if (!p.link) band();
     // the frame on fs
     if constexpr (DEV) {
-      if (p.n_frame)
-        kb_pml_fused<S><<<p.n_frame, 256, p.frame_smem, fs>>>(mem, p.frame_tab);
+      if (p.n_frame) {
+        const int* tab = p.frame_tab;
+        launch_begun(kb_pml_fused<S>, p.n_frame, 256, p.frame_smem, fs,
+                     aux && !p.n_f1 ? begun : nullptr, mem, tab);
+      }
     }
-    if (p.n_f1) kb_frame1<S, Real, DEV><<<p.n_f1, 128, 0, fs>>>(mem, p.f1_tab);
-    if (p.link) band();
-    if (p.n_f2) kb_frame2<S, Real><<<p.n_f2, 128, 0, fs>>>(mem, p.f2_tab);
+    launch_frame1(p, mem, fs, aux ? begun : nullptr);
+    if (aux && (p.n_frame || p.n_f1)) cudaStreamWaitEvent(st, begun, 0);
+    if (p.link) {
+      band();
+      if (fs != bs) {
+        cudaEventRecord(join, bs);
+        cudaStreamWaitEvent(fs, join, 0);
+      }
+    }
+    launch_frame2(p, mem, fs);
     // the interiors of every member on st
     if (p.n_bulk)
       kb_bulk<S, Real, DEV><<<p.n_bulk, dim3(p.tx, p.by),
