@@ -196,10 +196,9 @@ void nrbc_shape(const Geom& g, int* chunks, int* threads, size_t* smem) {
 }
 
 cudaError_t launch_nrbc_batch(const TgtDesc* d, const int* tab, int n, bool fp32, int threads,
-                              size_t smem, cudaStream_t s) {
+                              size_t smem, cudaStream_t s, cudaEvent_t begun) {
   if (n <= 0) return cudaSuccess;
-  if (fp32) kb_nrbc_rk4<float><<<n, threads, smem, s>>>(d, tab);
-  else kb_nrbc_rk4<double><<<n, threads, smem, s>>>(d, tab);
+  launch_begun(fp32 ? kb_nrbc_rk4<float> : kb_nrbc_rk4<double>, n, threads, smem, s, begun, d, tab);
   return cudaGetLastError();
 }
 

@@ -358,30 +358,6 @@ __global__ void __launch_bounds__(256) kb_wrap_y(const MemberDev<Real>* __restri
 // any size (128^2: 12.5 / 12.6 us).
 constexpr int kSplitBlocks = 256;
 
-// Launches `kernel` on s; `begun` (may be null) is an event that fires once all its blocks have
-// started. The interior waits for that event of the frame's first kernel: the frame, on the
-// critical path and short of blocks, goes first, and the interior fills the SMs as it drains.
-// Without it a graph starts the two in either order (link gradient, 1024^2, eight steps to a
-// graph: 162 us a step against 125; 512^2 printed 54 against 46, 2048^2 286 against 271).
-template <class... P, class... A>
-inline void launch_begun(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s,
-                         cudaEvent_t begun, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at = {};
-  if (begun) {
-    at.id = cudaLaunchAttributeLaunchCompletionEvent;
-    at.val.launchCompletionEvent.event = begun;
-    at.val.launchCompletionEvent.flags = 0;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-  }
-  cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 template <class S, class Real, bool DEV>
 struct Ops {
   static const Consts<Real>& consts(const Dev& d) {
@@ -451,8 +427,10 @@ struct Ops {
     const BatchPlan* pl = STREAM ? d.plan : nullptr;
     const MemberDev<Real>* pm = pl ? static_cast<const MemberDev<Real>*>(pl->desc[d.which]) : nullptr;
     if (pl) {
+      const cudaEvent_t begun = d.aux ? d.begun : nullptr;
       launch_nrbc_batch(pl->tgt[d.which], pl->tgt_tab, pl->n_tgt, sizeof(Real) == 4,
-                        pl->tgt_threads, pl->tgt_smem, bs);
+                        pl->tgt_threads, pl->tgt_smem, bs, begun);
+      if (begun && fs != bs && pl->n_tgt) cudaStreamWaitEvent(fs, begun, 0);
     } else if (STREAM && d.bc.bc == 2) {
       launch_nrbc_stages(d, sizeof(Real) == 4, bs);
     }
@@ -763,8 +741,9 @@ struct Ops {
     }
     // characteristic targets, then (printed gradient) the boundary band, on bs
     cudaError_t e = launch_nrbc_batch(p.tgt[which], p.tgt_tab, p.n_tgt, sizeof(Real) == 4,
-                                      p.tgt_threads, p.tgt_smem, bs);
+                                      p.tgt_threads, p.tgt_smem, bs, aux ? begun : nullptr);
     if (e != cudaSuccess) return e;
+    if (aux2 && p.n_tgt) cudaStreamWaitEvent(fs, begun, 0);
     auto band = [&]() { launch_band(p, mem, bs); };
     if (!p.link) band();
     // the frame on fs
