@@ -1326,32 +1326,6 @@ template <class R>
 struct PrimT { R rho, un, ut, T; };
 using Prim = PrimT<double>;
 
-// Inverse of the characteristic map: given w = S dU (acoustic-, entropy, shear, acoustic+),
-// return dU = S^-1 w in (rho, u_n, u_t, T). With P = rho T (c_s = 1), c^2 = 2 T (gamma = 2):
-// dP = (w1 + w4)/2, du_n = (w4 - w1)/(2 rho c), du_t = w3, drho = (dP + w2)/c^2,
-// dT = (dP - T drho)/rho.
-template <class R>
-__device__ inline PrimT<R> char_inverse(const PrimT<R>& U, R c, const R w[4]) {
-  PrimT<R> d;
-  const R dP = R(0.5) * (w[0] + w[3]);
-  d.un = (w[3] - w[0]) / (R(2) * U.rho * c);
-  d.ut = w[2];
-  d.rho = (dP + w[1]) / (c * c);
-  d.T = (dP - U.T * d.rho) / U.rho;
-  return d;
-}
-
-// w = S dU for the normal axis: w1 = T drho - rho c du_n + rho dT, w2 = T drho - rho dT,
-// w3 = du_t, w4 = T drho + rho c du_n + rho dT (left eigenvectors of the Euler Jacobian).
-template <class R>
-__device__ inline void char_forward(const PrimT<R>& U, R c, const PrimT<R>& dU, R w[4]) {
-  const R dP = U.T * dU.rho + U.rho * dU.T;
-  w[0] = dP - U.rho * c * dU.un;
-  w[1] = U.T * dU.rho - U.rho * dU.T;
-  w[2] = dU.ut;
-  w[3] = dP + U.rho * c * dU.un;
-}
-
 __device__ inline Prim load_prim(const double* V, int stride, int slot, bool xaxis) {
   Prim u;
   u.rho = V[slot];

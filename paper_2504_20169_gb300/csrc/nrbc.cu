@@ -10,52 +10,59 @@ namespace lbm {
 // the same layer around it along the tangent with weights (ca, cb, cc) of the tangential
 // derivative. PNR-LODI: Eq. (PNR) with Eq. (thermal_LODI_macro_evo); CBC relax: Eq. (CBC-Relax)
 // with Eq. (thermal_CBC_macro_evo); viscous part zero. Differences in FP64, algebra in R.
+//
+// The launch is one short chain, and each FP64 instruction in it costs 64 cycles: so one division
+// (1 / rho and 1 / (2 T) from 1 / (2 rho T)), factors that are powers of two applied to the sums in
+// R, and 1 / (rho c) as c / (rho c^2). With P = rho T, c^2 = 2 T (gamma = 2): wave amplitudes
+// w1,4 = T drho + rho dT -+ rho c du_n, w2 = T drho - rho dT, w3 = du_t, and back dP = (w1 + w4) / 2,
+// du_n = (w4 - w1) / (2 rho c), drho = (dP + w2) / c^2, dT = (dP - T drho) / rho. With five
+// divisions, FP64: 200 x 20 (D2Q17) 33.2 us a step, now 25.6; 300^2 51 -> 45 (FP32 within 2 %).
+// The four stages stay one loop that reads the fluid's nodes again: unrolled, with those in
+// registers (136 instead of 90), FP64 gains another 1 to 4 us, but the frame running beside it
+// loses more (FP32: 512^2 41 -> 50 us, 2048^2 270 -> 287).
 template <class R>
 __device__ inline void char_rate(const BcParams& bc, int variant, double out, const Prim& U0d,
                                  const Prim& U1, const Prim& U2, const Prim& Va, const Prim& Vb,
                                  const Prim& Vc, double ca, double cb, double cc, bool xaxis,
                                  double kk[4]) {
-  const double hs = 0.5 * out;
-  PrimT<R> dn;
-  dn.rho = R(hs * (3.0 * U0d.rho - 4.0 * U1.rho + U2.rho));
-  dn.un = R(hs * (3.0 * U0d.un - 4.0 * U1.un + U2.un));
-  dn.ut = R(hs * (3.0 * U0d.ut - 4.0 * U1.ut + U2.ut));
-  dn.T = R(hs * (3.0 * U0d.T - 4.0 * U1.T + U2.T));
+  auto normal = [](double u0, double u1, double u2) { return R(fma(-4.0, u1, fma(3.0, u0, u2))); };
   const PrimT<R> U0 = to<R>(U0d);
-  const R inv_r = R(bc.inv_r);
-  const R c = sqrt(R(2) * U0.T);  // gamma T with gamma = (D + 2) / D = 2
-  const R lam[4] = {U0.un - c, U0.un, U0.un, U0.un + c};
-  R wn[4];
-  char_forward(U0, c, dn, wn);
+  const R rho = U0.rho, un = U0.un, ut = U0.ut, T = U0.T;
+  const R T2 = T + T, c = sqrt(T2), rc = rho * c;
+  const R inv = R(1) / (rho * T2), irho = T2 * inv, iT2 = rho * inv;
   const R sgn = R(out);
-  R tot[4];
-  if (variant == 0) {
-    for (int k = 0; k < 4; ++k) tot[k] = (lam[k] * sgn < R(0)) ? R(0) : lam[k] * wn[k] * inv_r;
-  } else {
-    PrimT<R> dt;
-    dt.rho = R(ca * Va.rho + cb * Vb.rho + cc * Vc.rho);
-    dt.un = R(ca * Va.un + cb * Vb.un + cc * Vc.un);
-    dt.ut = R(ca * Va.ut + cb * Vb.ut + cc * Vc.ut);
-    dt.T = R(ca * Va.T + cb * Vb.T + cc * Vc.T);
-    // B dU along the tangential axis (u_t advects; P_t = T rho_t + rho T_t; (2/D) T = T)
-    PrimT<R> bd;
-    bd.rho = U0.ut * dt.rho + U0.rho * dt.ut;
-    bd.un = U0.ut * dt.un;
-    bd.ut = (U0.T / U0.rho) * dt.rho + U0.ut * dt.ut + dt.T;
-    bd.T = U0.T * dt.ut + U0.ut * dt.T;
-    R Tc[4];
-    char_forward(U0, c, bd, Tc);
-    const R relax = R(bc.relax_sign * (1.0 - bc.beta));
-    for (int k = 0; k < 4; ++k) {
-      const R Lbar = (lam[k] * sgn < R(0)) ? relax * Tc[k] : lam[k] * wn[k];
-      tot[k] = (Lbar + Tc[k]) * inv_r;
-    }
+  const bool in0 = (un - c) * sgn < R(0), in1 = un * sgn < R(0), in3 = (un + c) * sgn < R(0);
+  R t0, t1, t2, t3;   // lambda_k w_k of the normal differences, in units of out / (2 r)
+  {
+    const R a = T * normal(U0d.rho, U1.rho, U2.rho), b = rho * normal(U0d.T, U1.T, U2.T);
+    const R g = rc * normal(U0d.un, U1.un, U2.un);
+    t0 = in0 ? R(0) : (un - c) * (a + b - g);
+    t1 = in1 ? R(0) : un * (a - b);
+    t2 = in1 ? R(0) : un * normal(U0d.ut, U1.ut, U2.ut);
+    t3 = in3 ? R(0) : (un + c) * (a + b + g);
   }
-  const PrimT<R> r = char_inverse(U0, c, tot);
-  kk[0] = -double(r.rho);
-  kk[1] = xaxis ? -double(r.un) : -double(r.ut);
-  kk[2] = xaxis ? -double(r.ut) : -double(r.un);
-  kk[3] = -double(r.T);
+  R scale = R(0.5 * out * bc.inv_r);
+  if (variant != 0) {
+    // B dU along the tangential axis (u_t advects; P_t = T rho_t + rho T_t; (2/D) T = T)
+    auto along = [&](double va, double vb, double vc) { return R(ca * va + cb * vb + cc * vc); };
+    const R dr = along(Va.rho, Vb.rho, Vc.rho), dn = along(Va.un, Vb.un, Vc.un);
+    const R dt = along(Va.ut, Vb.ut, Vc.ut), dT = along(Va.T, Vb.T, Vc.T);
+    const R br = ut * dr + rho * dt, bT = T * dt + ut * dT;
+    const R a = T * br, b = rho * bT, g = rc * (ut * dn);
+    const R w0 = a + b - g, w1 = a - b, w2 = T * irho * dr + ut * dt + dT, w3 = a + b + g;
+    const R relax = R(1.0 + bc.relax_sign * (1.0 - bc.beta)), h = R(0.5 * out);
+    t0 = in0 ? relax * w0 : h * t0 + w0;
+    t1 = in1 ? relax * w1 : h * t1 + w1;
+    t2 = in1 ? relax * w2 : h * t2 + w2;
+    t3 = in3 ? relax * w3 : h * t3 + w3;
+    scale = R(bc.inv_r);
+  }
+  const R dP = R(0.5) * (t0 + t3), drho = (dP + t1) * iT2;
+  const R run = R(0.5) * (t3 - t0) * (c * inv), rT = (dP - T * drho) * irho;
+  kk[0] = -double(scale * drho);
+  kk[1] = -double(scale * (xaxis ? run : t2));
+  kk[2] = -double(scale * (xaxis ? t2 : run));
+  kk[3] = -double(scale * rT);
 }
 
 // All four stages of classical RK4 for the targets of one chunk of one edge band, in shared
