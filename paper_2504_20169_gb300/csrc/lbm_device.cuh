@@ -6,6 +6,9 @@
 // boundary. In LBM_FP32_DEV storage each value is g_i = f_i - w_i (deviation from the rest
 // state), otherwise the absolute f_i in FP64.
 //
+// FP64 nodes are updated in 64-bit fixed point (fixed.cuh) where their state allows it, by the same
+// kernels; the floating-point bodies serve FP32 and the FP64 states outside that range.
+//
 // A stored buffer always holds post-collision populations f* of one time level; a step pulls
 // f^(n+1)(x) = f*^n(x - e_i) (Eq. lbe), collides, and writes f*^(n+1).
 //
@@ -884,7 +887,11 @@ __device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c
   const PmlLayers<Real> pn = pml_layers(g, c, x, y);
   if (!pn.in_p) return;
   const Real sx = pn.sx, sy = pn.sy;
-  if (g.link) {
+  // STAGE: the FP32 kernel, which only the link gradient launches (the printed one has its frame in
+  // one kernel). Without the printed form beside it the compiler keeps the addresses of the stores
+  // (124 registers instead of 106, still four blocks an SM): the batched sweep of 16 members
+  // 1056 -> 1005 us a step.
+  if (STAGE || g.link) {
     // link mode: the remaining -sigma Q_i(x + e_i) of -sigma (Q_i(x + e_i) - Q_i(x)), the
     // integral of sigma c_i . grad Q_i along the link the population travels (sigma_x =
     // sigma_y); phase 1 added +sigma Q_i(x), and Q^n sits in the S^(n-1) slots of the frame and
