@@ -358,6 +358,13 @@ __global__ void __launch_bounds__(256) kb_wrap_y(const MemberDev<Real>* __restri
 // any size (128^2: 12.5 / 12.6 us).
 constexpr int kSplitBlocks = 256;
 
+// Tiles of the fused FP32 frame up to which the interior waits for the frame's last block to start
+// (launch_begun): twelve waves of two blocks to each of 152 SMs. Beyond, that wait costs more than
+// the order gives (us a step, waiting / not: 2430 tiles, 4096^2 + PML 32, 895 / 900; 3640, 3072^2 +
+// 64, 645 / 643; 4830, 4096^2 + 64, 1044 / 1032; 9570, 8192^2 + 64, 3571 / 3501). A batch, whose
+// interiors are small beside its frames, always waits (16 members, 5000 tiles, 847 / 858).
+constexpr int kFrameFirst = 12 * 304;
+
 template <class S, class Real, bool DEV>
 struct Ops {
   static const Consts<Real>& consts(const Dev& d) {
@@ -437,7 +444,7 @@ struct Ops {
     mark(1, bs);
     mark(4, fs);
     if (pl) {
-      const cudaEvent_t begun = d.aux ? d.begun : nullptr;
+      const cudaEvent_t begun = d.aux && pl->n_frame <= kFrameFirst ? d.begun : nullptr;
       if constexpr (DEV) {
         if (pl->n_frame) {
           const int* tab = pl->frame_tab;
