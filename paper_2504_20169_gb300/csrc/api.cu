@@ -571,8 +571,6 @@ lbm_status lbm_create(const lbm_grid* grid, lbm_stencil stencil, double tau, int
   d.flag = ctx->dflag;
   d.Vtgt = ctx->V;
   d.Va = ctx->V + 4 * (size_t)g.nb;
-  d.Vb = ctx->V + 8 * (size_t)g.nb;
-  d.Vacc = ctx->V + 12 * (size_t)g.nb;
   d.bc.bc = (int)bc;
   for (int k = 0; k < 4; ++k) d.bc.edge[k] = bp.edge[k];
   d.bc.beta = bp.beta;

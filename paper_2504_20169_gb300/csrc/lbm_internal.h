@@ -19,9 +19,7 @@ struct Dev {
   void* Sold;        // PML accumulator S^(n-1) (link mode: Q^n in place during the step)
   void* Snew;        // S^n
   double* Vtgt;      // characteristic targets U_tgt [4][nb]
-  double* Va;        // Runge-Kutta stage buffers [4][nb]
-  double* Vb;
-  double* Vacc;
+  double* Va;        // the rest of that allocation, [12][nb]; its start holds the sigma table
   // fluid moments of the outer two layers of F [4][ne], two buffers: the characteristic
   // targets read the level-n moments (Uedge_in, written by the previous step's frame) while
   // this step's frame writes the next level's (Uedge_out), so the two can run concurrently

@@ -1,5 +1,6 @@
-// Vector FMA throughput of the current device (lbm_peak_fma in lbm.h): the ALU roofline of
-// the FP64 path, whose interior kernel is bound by the FP64 pipe rather than by HBM.
+// Vector FMA throughput of the current device (lbm_peak_fma in lbm.h): what the
+// FP64 path's rate is reported against. Its node updates run in 64-bit fixed point, because this
+// pipe's FP64 rate would bound them (fixed.cuh).
 //
 // Every thread runs eight independent fused multiply-add chains a = a * b + c (enough
 // independent work per warp to keep the pipe busy); the grid fills every SM to its thread

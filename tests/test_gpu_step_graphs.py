@@ -1,0 +1,61 @@
+"""How a step is launched does not change what it computes: graphs of eight steps, the steps
+before and after them, and the kernels that put four warps to 32 FP64 nodes on small launches."""
+import numpy as np
+import pytest
+
+import workloads as wl
+from parity_helpers import case_kwargs, make_solver
+
+pytestmark = pytest.mark.gpu
+
+
+def populations(kw, prec, fields, calls):
+    with make_solver(kw, prec) as s:
+        s.init(*fields)
+        for n in calls:
+            s.step(n)
+        s.sync()
+        return s.export_populations()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32dev"])
+@pytest.mark.parametrize("q,bc,grad,W", [(37, "nrbc", "central", 5), (37, "nrbc", "link", 5),
+                                         (17, "nrbc", "central", 4), (9, "zg", "link", 3),
+                                         (17, "periodic", "central", 0)])
+def test_many_steps_equal_single_steps(prec, q, bc, grad, W):
+    """step(n) below, at and beyond a graph's length, from both buffer parities, against step(1)."""
+    kw = case_kwargs(nx=45, ny=37, W=W, tau=0.8, sigma_max=0.05 if W else 0.0, sigma_power=2, bc=bc,
+                     q=q, pml_grad=grad, mean=(1.0, 0.1, 0.05, 1.0))
+    f = wl.random_smooth_state(45, 37, W, seed=q, du=0.02, drho=0.01, dT=0.01, mean_u=(0.1, 0.05))
+    ref = populations(kw, prec, f, [1] * 30)
+    for calls in ([30], [1, 8, 21], [3, 16, 11], [7, 17, 6], [5] * 6):
+        assert np.array_equal(populations(kw, prec, f, calls), ref)
+
+
+@pytest.mark.parametrize("q,grad", [(37, "central"), (17, "link"), (9, "central")])
+def test_large_fp64_batch_equals_its_members(q, grad):
+    """A batch with more blocks than the split kernels take against members alone, which they do."""
+    import torch
+
+    from paper_2504_20169_gb300.serving import Batch
+
+    nx, ny, W, n = 96, 80, 8, 14      # 14 x 24 frame blocks of 128 nodes
+    kw = case_kwargs(nx=nx, ny=ny, W=W, tau=0.8, sigma_max=0.05, sigma_power=2, bc="nrbc", q=q,
+                     pml_grad=grad, mean=(1.0, 0.1, 0.0, 1.0))
+    states = [wl.random_smooth_state(nx, ny, W, seed=m, du=0.02, drho=0.01, dT=0.01,
+                                     mean_u=(0.1, 0.0)) for m in range(n)]
+    solvers = [make_solver(kw, "fp64") for _ in range(n)]
+    try:
+        for s, f in zip(solvers, states):
+            s.init(*f)
+        batch = Batch()
+        batch.set(solvers)
+        batch.step(11)
+        torch.cuda.synchronize()
+        batch.close()
+        got = [s.export_populations() for s in solvers]
+    finally:
+        for s in solvers:
+            s.close()
+    for m in range(n):
+        assert np.array_equal(got[m], populations(kw, "fp64", states[m], [11]))
