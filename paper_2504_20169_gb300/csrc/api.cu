@@ -206,7 +206,8 @@ struct lbm_ctx {
   cudaStream_t st = nullptr;
   void* f[2] = {nullptr, nullptr};
   void* S[2] = {nullptr, nullptr};
-  double* V = nullptr;        // 4 arrays of [4][nb]: targets, stage a, stage b, accumulator
+  double* V = nullptr;        // targets, two buffers of [4][nb] (ping-pong with the populations);
+                              // then the sigma table
   double* Uedge = nullptr;    // two buffers of [4][ne] (ping-pong with the populations)
   double* Sedge = nullptr;    // two buffers of [4][2 (Lx + Ly)]: Appendix PML source
   double* staging = nullptr;  // [4][Lx*Ly]
@@ -301,6 +302,7 @@ constexpr int kGraphSteps = 8, kDirectSteps = 4;
 // of host time each, before a context builds the graphs of one step (35 us each, 5 us a launch).
 constexpr int kSingles = 16;
 
+static size_t target_slots(const Geom& g) { return 4 * (size_t)g.nb; }
 static size_t edge_slots(const Geom& g) { return 4 * (size_t)g.ne; }
 static size_t source_slots(const Geom& g) { return 4 * 2 * ((size_t)g.Lx + g.Ly); }
 
@@ -311,6 +313,8 @@ static void set_roles(lbm_ctx* ctx, int a, int s) {
   d.B = ctx->f[1 - a];
   d.Sold = ctx->S[s];
   d.Snew = ctx->S[1 - s];
+  d.Vtgt_in = ctx->V + a * target_slots(ctx->g);
+  d.Vtgt = ctx->V + (1 - a) * target_slots(ctx->g);
   d.Uedge_in = ctx->Uedge + a * edge_slots(ctx->g);
   d.Uedge_out = ctx->Uedge + (1 - a) * edge_slots(ctx->g);
   d.Sedge_in = ctx->Sedge + a * source_slots(ctx->g);
@@ -569,8 +573,6 @@ lbm_status lbm_create(const lbm_grid* grid, lbm_stencil stencil, double tau, int
   d.join2 = ctx->join2;
   d.begun = ctx->begun;
   d.flag = ctx->dflag;
-  d.Vtgt = ctx->V;
-  d.Va = ctx->V + 4 * (size_t)g.nb;
   d.bc.bc = (int)bc;
   for (int k = 0; k < 4; ++k) d.bc.edge[k] = bp.edge[k];
   d.bc.beta = bp.beta;
@@ -600,8 +602,9 @@ lbm_status lbm_create(const lbm_grid* grid, lbm_stencil stencil, double tau, int
   d.cf.sigma_max = (float)sg.sigma_max; d.cf.power = sg.power; d.cf.split = sg.split;
   {
     // sigma of every layer of the W, E, S and N edge (index 0: none), as sigma_of forms it, in the
-    // part of the target buffer that the fused Runge-Kutta launch leaves free (12 M (Lx + Ly) or
-    // more doubles against at most Lx + Ly + 4)
+    // part of the targets' allocation behind the two buffers (16 M (Lx + Ly) doubles against at
+    // most Lx + Ly + 4)
+    double* const table = ctx->V + 2 * target_slots(g);
     std::vector<double> sd;
     std::vector<float> sf;
     for (int e = 0; e < 4; ++e)
@@ -616,12 +619,12 @@ lbm_status lbm_create(const lbm_grid* grid, lbm_stencil stencil, double tau, int
         sf.push_back(i ? d.cf.sigma_max * pf : 0.0f);
       }
     const bool f32 = precision == LBM_FP32_DEV;
-    if (cudaMemcpyAsync(d.Va, f32 ? (const void*)sf.data() : (const void*)sd.data(),
+    if (cudaMemcpyAsync(table, f32 ? (const void*)sf.data() : (const void*)sd.data(),
                         f32 ? sf.size() * sizeof(float) : sd.size() * sizeof(double),
                         cudaMemcpyHostToDevice, ctx->st) != cudaSuccess)
       return oom("sigma table");
-    d.cd.sigma = d.Va;
-    d.cf.sigma = reinterpret_cast<const float*>(d.Va);
+    d.cd.sigma = table;
+    d.cf.sigma = reinterpret_cast<const float*>(table);
   }
   if (ctx->ops.prepare(ctx->w) != cudaSuccess) return oom("kernel attributes");
   {
@@ -1045,7 +1048,9 @@ lbm_status lbm_checkpoint(lbm_ctx* ctx, void* host, size_t bytes) {
   LBM_CK(cudaMemcpyAsync(p, ctx->f[ctx->cur], ctx->fbytes, k, ctx->st)); p += ctx->fbytes;
   LBM_CK(cudaMemcpyAsync(p, ctx->f[1 - ctx->cur], ctx->fbytes, k, ctx->st)); p += ctx->fbytes;
   if (ctx->sbytes) { LBM_CK(cudaMemcpyAsync(p, ctx->S[ctx->scur], ctx->sbytes, k, ctx->st)); p += ctx->sbytes; }
-  LBM_CK(cudaMemcpyAsync(p, ctx->V, sizeof(double) * 4 * ctx->g.nb, k, ctx->st)); p += sizeof(double) * 4 * ctx->g.nb;
+  LBM_CK(cudaMemcpyAsync(p, ctx->V + ctx->cur * target_slots(ctx->g),
+                         sizeof(double) * target_slots(ctx->g), k, ctx->st));
+  p += sizeof(double) * target_slots(ctx->g);
   // the edge moments the next step's targets read
   LBM_CK(cudaMemcpyAsync(p, ctx->Uedge + ctx->cur * edge_slots(ctx->g),
                          sizeof(double) * edge_slots(ctx->g), k, ctx->st));
@@ -1078,7 +1083,8 @@ lbm_status lbm_restore(lbm_ctx* ctx, const void* host, size_t bytes) {
   LBM_CK(cudaMemcpyAsync(ctx->f[0], p, ctx->fbytes, k, ctx->st)); p += ctx->fbytes;
   LBM_CK(cudaMemcpyAsync(ctx->f[1], p, ctx->fbytes, k, ctx->st)); p += ctx->fbytes;
   if (ctx->sbytes) { LBM_CK(cudaMemcpyAsync(ctx->S[0], p, ctx->sbytes, k, ctx->st)); p += ctx->sbytes; }
-  LBM_CK(cudaMemcpyAsync(ctx->V, p, sizeof(double) * 4 * ctx->g.nb, k, ctx->st)); p += sizeof(double) * 4 * ctx->g.nb;
+  LBM_CK(cudaMemcpyAsync(ctx->V, p, sizeof(double) * target_slots(ctx->g), k, ctx->st));
+  p += sizeof(double) * target_slots(ctx->g);
   LBM_CK(cudaMemcpyAsync(ctx->Uedge, p, sizeof(double) * edge_slots(ctx->g), k, ctx->st));
   p += sizeof(double) * edge_slots(ctx->g);
   LBM_CK(cudaMemcpyAsync(ctx->Sedge, p, sizeof(double) * source_slots(ctx->g), k, ctx->st));

@@ -18,8 +18,10 @@ struct Dev {
   void* B;           // next level (written)
   void* Sold;        // PML accumulator S^(n-1) (link mode: Q^n in place during the step)
   void* Snew;        // S^n
-  double* Vtgt;      // characteristic targets U_tgt [4][nb]
-  double* Va;        // the rest of that allocation, [12][nb]; its start holds the sigma table
+  // characteristic targets U_tgt [4][nb], two buffers: a chunk of an edge band also reads its
+  // neighbours' targets of level n (Vtgt_in), so those of level n + 1 go to the other one (Vtgt)
+  const double* Vtgt_in;
+  double* Vtgt;
   // fluid moments of the outer two layers of F [4][ne], two buffers: the characteristic
   // targets read the level-n moments (Uedge_in, written by the previous step's frame) while
   // this step's frame writes the next level's (Uedge_out), so the two can run concurrently
@@ -54,6 +56,7 @@ struct TgtDesc {
   BcParams bc;
   const double* Ue;
   const double* Se;
+  const double* Vin;
   double* V;
 };
 

@@ -66,7 +66,9 @@ __device__ inline void char_rate(const BcParams& bc, int variant, double out, co
 }
 
 // All four stages of classical RK4 for the targets of one chunk of one edge band, in shared
-// memory (fluid moments Ue frozen at time n). Block = one edge, tangential chunk [t0, t0 + T)
+// memory (fluid moments Ue frozen at time n), from the targets Vin of level n to V of level n + 1:
+// two arrays, because blocks run in any order and a block's halo is another block's chunk.
+// Block = one edge, tangential chunk [t0, t0 + T)
 // plus a 4-node halo on each side where the chunk does not end the band; thread = (layer,
 // position). Each stage shrinks the valid range by one node at a chunk cut, so the chunk's own
 // nodes see exactly the values a full-band evaluation would. On a periodic y axis the W and E
@@ -79,7 +81,8 @@ template <class R>
 __device__ __forceinline__ void nrbc_chunk(const Geom& g, const BcParams& bc,
                                            const double* __restrict__ Ue,
                                            const double* __restrict__ Se,
-                                           double* __restrict__ Vg, int chunk, double* sm) {
+                                           const double* __restrict__ Vin,
+                                           double* __restrict__ V, int chunk, double* sm) {
   const int M = g.M, Lx = g.Lx, Ly = g.Ly;
   const int cw = (Ly + kChunk - 1) / kChunk, cs = (Lx + kChunk - 1) / kChunk;
   int e, k = chunk;
@@ -108,7 +111,7 @@ __device__ __forceinline__ void nrbc_chunk(const Geom& g, const BcParams& bc,
   const int j = tid / kText + 1, t = lo + tid % kText;
   const bool live = j <= M && t < hi;
   if (live)
-    for (int q = 0; q < 4; ++q) at(0, q, j, t) = Vg[q * g.nb + off + (j - 1) * len + wr(t)];
+    for (int q = 0; q < 4; ++q) at(0, q, j, t) = Vin[q * g.nb + off + (j - 1) * len + wr(t)];
   __syncthreads();
   auto prim = [&](int buf, int jj, int tt) {
     Prim u;
@@ -174,7 +177,7 @@ __device__ __forceinline__ void nrbc_chunk(const Geom& g, const BcParams& bc,
       } else if (t >= t0 && t < t0 + kChunk && t < len) {
         const double sixth = 1.0 / 6.0;
         for (int q = 0; q < 4; ++q)
-          Vg[q * g.nb + off + (j - 1) * len + t] = at(0, q, j, t) + (at(3, q, j, t) + kk[q]) * sixth;
+          V[q * g.nb + off + (j - 1) * len + t] = at(0, q, j, t) + (at(3, q, j, t) + kk[q]) * sixth;
       }
     }
     __syncthreads();
@@ -183,9 +186,10 @@ __device__ __forceinline__ void nrbc_chunk(const Geom& g, const BcParams& bc,
 
 template <class R>
 __global__ void k_nrbc_rk4(Geom g, BcParams bc, const double* __restrict__ Ue,
-                           const double* __restrict__ Se, double* __restrict__ Vg) {
+                           const double* __restrict__ Se, const double* __restrict__ Vin,
+                           double* __restrict__ V) {
   extern __shared__ double sm[];
-  nrbc_chunk<R>(g, bc, Ue, Se, Vg, blockIdx.x, sm);
+  nrbc_chunk<R>(g, bc, Ue, Se, Vin, V, blockIdx.x, sm);
 }
 
 template <class R>
@@ -193,7 +197,7 @@ __global__ void kb_nrbc_rk4(const TgtDesc* __restrict__ d, const int* __restrict
   extern __shared__ double sm[];
   const int m = tab[2 * blockIdx.x], chunk = tab[2 * blockIdx.x + 1];
   const TgtDesc& t = d[m];
-  nrbc_chunk<R>(t.g, t.bc, t.Ue, t.Se, t.V, chunk, sm);
+  nrbc_chunk<R>(t.g, t.bc, t.Ue, t.Se, t.Vin, t.V, chunk, sm);
 }
 
 void nrbc_shape(const Geom& g, int* chunks, int* threads, size_t* smem) {
@@ -217,9 +221,11 @@ cudaError_t launch_nrbc_stages(const Dev& d, bool fp32, cudaStream_t s) {
   size_t smem;
   nrbc_shape(g, &blocks, &threads, &smem);
   if (fp32)
-    k_nrbc_rk4<float><<<blocks, threads, smem, s>>>(g, d.bc, d.Uedge_in, d.Sedge_in, d.Vtgt);
+    k_nrbc_rk4<float><<<blocks, threads, smem, s>>>(g, d.bc, d.Uedge_in, d.Sedge_in, d.Vtgt_in,
+                                                    d.Vtgt);
   else
-    k_nrbc_rk4<double><<<blocks, threads, smem, s>>>(g, d.bc, d.Uedge_in, d.Sedge_in, d.Vtgt);
+    k_nrbc_rk4<double><<<blocks, threads, smem, s>>>(g, d.bc, d.Uedge_in, d.Sedge_in, d.Vtgt_in,
+                                                     d.Vtgt);
   return cudaGetLastError();
 }
 

@@ -699,8 +699,10 @@ struct Ops {
     for (int m = 0; m < n; ++m) {
       d0[m] = member_of(*dev0[m]);
       d1[m] = member_of(*dev1[m]);
-      t0[m] = TgtDesc{dev0[m]->g, dev0[m]->bc, dev0[m]->Uedge_in, dev0[m]->Sedge_in, dev0[m]->Vtgt};
-      t1[m] = TgtDesc{dev1[m]->g, dev1[m]->bc, dev1[m]->Uedge_in, dev1[m]->Sedge_in, dev1[m]->Vtgt};
+      t0[m] = TgtDesc{dev0[m]->g, dev0[m]->bc, dev0[m]->Uedge_in, dev0[m]->Sedge_in,
+                      dev0[m]->Vtgt_in, dev0[m]->Vtgt};
+      t1[m] = TgtDesc{dev1[m]->g, dev1[m]->bc, dev1[m]->Uedge_in, dev1[m]->Sedge_in,
+                      dev1[m]->Vtgt_in, dev1[m]->Vtgt};
     }
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t bd = al(sizeof(MemberDev<Real>) * n), bt = al(sizeof(TgtDesc) * n);
