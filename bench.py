@@ -666,7 +666,7 @@ def main():
             "serving_sustainable": serving_sustainable,
             "variants_fp32": variants, "long_run_fp32": longrun,
             "e2e": e2e, "cpu_baseline": cpu,
-            # per step: k_nrbc_rk4, k_pml_fused, k_gamma, k_bulk (one CUDA-graph replay); the
+            # per step: kb_nrbc_rk4, kb_pml_fused, kb_gamma, k_bulk (one CUDA-graph replay); the
             # link gradient runs the frame as two kernels
             "gpu_launches": args.steps * ((4 if c.bc == "nrbc" else 3) + (c.pml_grad == "link")),
             "clocks": ck,

@@ -12,8 +12,10 @@
 // A stored buffer always holds post-collision populations f* of one time level; a step pulls
 // f^(n+1)(x) = f*^n(x - e_i) (Eq. lbe), collides, and writes f*^(n+1).
 //
-// Work split of one step (all kernels read buffer A and write disjoint parts of buffer B):
-//   k_nrbc_rk4        characteristic targets U_tgt^(n+1) on the edge bands, four RK4 stages (Sec. 4)
+// Work split of one step (all kernels read buffer A and write disjoint parts of buffer B). Streaming
+// steps run the table-driven form kb_* of each (ops.cuh), the collision of the initial state the k_*
+// named here; the interior of a context alone is k_bulk in both.
+//   kb_nrbc_rk4       characteristic targets U_tgt^(n+1) on the edge bands, four RK4 stages (Sec. 4)
 //   k_bulk            nodes of F inside the frame depths (Fw, Fe, Fs, Fn): BGK only
 //   k_frame1          the frame (the outer Fw / Fe / Fs / Fn layers of F): BGK, PML
 //                     accumulator, local PML terms,
@@ -859,16 +861,17 @@ constexpr int edge_blocks() {
   return sizeof(Real) == 4 ? 0 : S::Q == 37 ? 4 : S::Q == 17 ? 5 : 8;
 }
 
-template <class S, class Real, bool DEV, bool STREAM>
+// The initial state's frame (streaming steps: kb_frame1).
+template <class S, class Real, bool DEV>
 __global__ void __launch_bounds__(128, edge_blocks<S, Real>()) k_frame1(
     const __grid_constant__ Geom g, const __grid_constant__ Consts<Real> c,
-                                                const Real* __restrict__ A, Real* __restrict__ B, Real* __restrict__ Sold,
-                                                Real* __restrict__ Snew, double* Uedge, int save_edges,
-                                                int* flag, double* Sedge, int src_mask) {
+    const Real* __restrict__ A, Real* __restrict__ B, Real* __restrict__ Sold,
+    Real* __restrict__ Snew, double* Uedge, int save_edges, int* flag, double* Sedge,
+    int src_mask) {
   __shared__ double f[node_smem<S, Real>(128)];
-  frame1_node<S, Real, DEV, STREAM>(g, c, A, B, Sold, Snew, Uedge, save_edges, flag, Sedge,
-                                    src_mask, blockIdx.x * blockDim.x + threadIdx.x,
-                                    reinterpret_cast<Real*>(f) + threadIdx.x, 128);
+  frame1_node<S, Real, DEV, false>(g, c, A, B, Sold, Snew, Uedge, save_edges, flag, Sedge,
+                                   src_mask, blockIdx.x * blockDim.x + threadIdx.x,
+                                   reinterpret_cast<Real*>(f) + threadIdx.x, 128);
 }
 
 // Frame, phase 2 (PML nodes): subtract sigma_y c_ix dQ_i/dx + sigma_x c_iy dQ_i/dy (sigma
@@ -1294,16 +1297,15 @@ __device__ __forceinline__ void gamma_split(const Geom& g, const Consts<double>&
     gamma_outside<S, true>(g, c, bc, A, B, Vtgt, b, Sold, Snew, t, src, dst);
 }
 
-template <class S, class Real, bool DEV, bool STREAM>
+// The initial state's band (streaming steps: kb_gamma).
+template <class S, class Real, bool DEV>
 __global__ void __launch_bounds__(128, edge_blocks<S, Real>()) k_gamma(
     const __grid_constant__ Geom g, const __grid_constant__ Consts<Real> c,
     const __grid_constant__ BcParams bc, const Real* __restrict__ A, Real* __restrict__ B,
-                                               const double* __restrict__ Vtgt,
-                                               Real* __restrict__ Sold,
-                                               Real* __restrict__ Snew) {
+    const double* __restrict__ Vtgt, Real* __restrict__ Sold, Real* __restrict__ Snew) {
   __shared__ double f[node_smem<S, Real>(128)];
-  gamma_node<S, Real, DEV, STREAM>(g, c, bc, A, B, Vtgt, Sold, Snew,
-                                   blockIdx.x * blockDim.x + threadIdx.x, f + threadIdx.x, 128);
+  gamma_node<S, Real, DEV, false>(g, c, bc, A, B, Vtgt, Sold, Snew,
+                                  blockIdx.x * blockDim.x + threadIdx.x, f + threadIdx.x, 128);
 }
 
 // Periodic y axis: the M rows below y = 0 and above y = Ly - 1 (boundary columns included)

@@ -135,7 +135,8 @@ void batch_plan_free(BatchPlan* plan);
 // block, dynamic shared memory.
 void nrbc_shape(const Geom& g, int* chunks, int* threads, size_t* smem);
 
-// Batched characteristic targets: one block per table entry (member, chunk).
+// Characteristic targets: one block per table entry (member, chunk); fp32 selects FP32
+// characteristic algebra (targets and differences stay FP64).
 cudaError_t launch_nrbc_batch(const TgtDesc* d, const int* tab, int n, bool fp32, int threads,
                               size_t smem, cudaStream_t s, cudaEvent_t begun);
 
@@ -145,10 +146,6 @@ OpsTable ops_q17_f64();
 OpsTable ops_q17_f32();
 OpsTable ops_q9_f64();
 OpsTable ops_q9_f32();
-
-// Characteristic-target RK4 stages of one step on stream s; fp32 selects FP32 characteristic
-// algebra (targets and differences stay FP64).
-cudaError_t launch_nrbc_stages(const Dev& d, bool fp32, cudaStream_t s);
 
 // Message returned by lbm_last_error(NULL) (calls without a context).
 void set_global_error(const std::string& msg);

@@ -75,8 +75,7 @@ __device__ inline void char_rate(const BcParams& bc, int variant, double out, co
 // bands wrap around (central tangential differences everywhere, halo taken modulo Ly).
 constexpr int kChunk = 32, kHalo = 4, kText = kChunk + 2 * kHalo;
 
-// (nrbc_chunk is the per-block work, shared with the batched launch over many instances;
-// chunk = index over the four bands' chunks, sm = 16 M kText doubles of shared memory.)
+// (nrbc_chunk is the per-block work; chunk = index over the four bands' chunks, sm = 16 M kText doubles of shared memory.)
 template <class R>
 __device__ __forceinline__ void nrbc_chunk(const Geom& g, const BcParams& bc,
                                            const double* __restrict__ Ue,
@@ -185,14 +184,6 @@ __device__ __forceinline__ void nrbc_chunk(const Geom& g, const BcParams& bc,
 }
 
 template <class R>
-__global__ void k_nrbc_rk4(Geom g, BcParams bc, const double* __restrict__ Ue,
-                           const double* __restrict__ Se, const double* __restrict__ Vin,
-                           double* __restrict__ V) {
-  extern __shared__ double sm[];
-  nrbc_chunk<R>(g, bc, Ue, Se, Vin, V, blockIdx.x, sm);
-}
-
-template <class R>
 __global__ void kb_nrbc_rk4(const TgtDesc* __restrict__ d, const int* __restrict__ tab) {
   extern __shared__ double sm[];
   const int m = tab[2 * blockIdx.x], chunk = tab[2 * blockIdx.x + 1];
@@ -210,22 +201,6 @@ cudaError_t launch_nrbc_batch(const TgtDesc* d, const int* tab, int n, bool fp32
                               size_t smem, cudaStream_t s, cudaEvent_t begun) {
   if (n <= 0) return cudaSuccess;
   launch_begun(fp32 ? kb_nrbc_rk4<float> : kb_nrbc_rk4<double>, n, threads, smem, s, begun, d, tab);
-  return cudaGetLastError();
-}
-
-// The four RK4 stages of one step in one launch; fp32 selects FP32 characteristic algebra
-// (targets and differences stay FP64).
-cudaError_t launch_nrbc_stages(const Dev& d, bool fp32, cudaStream_t s) {
-  const Geom& g = d.g;
-  int blocks, threads;
-  size_t smem;
-  nrbc_shape(g, &blocks, &threads, &smem);
-  if (fp32)
-    k_nrbc_rk4<float><<<blocks, threads, smem, s>>>(g, d.bc, d.Uedge_in, d.Sedge_in, d.Vtgt_in,
-                                                    d.Vtgt);
-  else
-    k_nrbc_rk4<double><<<blocks, threads, smem, s>>>(g, d.bc, d.Uedge_in, d.Sedge_in, d.Vtgt_in,
-                                                     d.Vtgt);
   return cudaGetLastError();
 }
 

@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <utility>
 #include <vector>
 
 #include "lbm_device.cuh"
@@ -404,122 +405,19 @@ struct Ops {
     kb_gamma<S, Real, DEV><<<p.n_band, 128, 0, s>>>(m, p.band_tab);
   }
 
-  template <bool STREAM>
-  static cudaError_t step_impl(const Dev& d) {
-    const Geom& g = d.g;
-    const Consts<Real>& c = consts(d);
-    const Real* A = static_cast<const Real*>(d.A);
-    Real* B = static_cast<Real*>(d.B);
-    // characteristic targets then boundary band on bs, PML frame on fs, interior on d.st; all
-    // read A and write disjoint parts of B
-    const bool link = g.link && has_pml(g);
-    const cudaStream_t bs = d.aux ? d.aux : d.st;
-    // link mode: the gradient pass reads the boundary nodes' new accumulator, so phase 2 of the
-    // frame waits for the band
-    const cudaStream_t fs = d.aux2 ? d.aux2 : bs;
-    auto mark = [&](int k, cudaStream_t s) {
-      if (d.ev) cudaEventRecord(d.ev[k], s);
-    };
+  // Boundary-side work forks from d.st: the boundary band on the first stream returned, the PML
+  // frame on the second; both join d.st again in join_streams. All read A and write disjoint parts
+  // of B.
+  static std::pair<cudaStream_t, cudaStream_t> fork_streams(const Dev& d) {
     if (d.aux) {
       cudaEventRecord(d.fork, d.st);
       cudaStreamWaitEvent(d.aux, d.fork, 0);
       if (d.aux2) cudaStreamWaitEvent(d.aux2, d.fork, 0);
     }
-    // Appendix PML source terms: only with a characteristic BC and a PML
-    const int src_mask = (d.bc.bc == 2 && has_pml(g)) ? (d.bc.pml_source & 7) : 0;
-    mark(0, bs);
-    // Streaming steps of a context run the boundary-side classes through the table-driven
-    // kernels of its one-member plan (the kernels a batch runs), so that a context computes
-    // bit for bit the same alone and in any batch; the interior kernel is the same either way.
-    const BatchPlan* pl = STREAM ? d.plan : nullptr;
-    const MemberDev<Real>* pm = pl ? static_cast<const MemberDev<Real>*>(pl->desc[d.which]) : nullptr;
-    if (pl) {
-      const cudaEvent_t begun = d.aux ? d.begun : nullptr;
-      launch_nrbc_batch(pl->tgt[d.which], pl->tgt_tab, pl->n_tgt, sizeof(Real) == 4,
-                        pl->tgt_threads, pl->tgt_smem, bs, begun);
-      if (begun && fs != bs && pl->n_tgt) cudaStreamWaitEvent(fs, begun, 0);
-    } else if (STREAM && d.bc.bc == 2) {
-      launch_nrbc_stages(d, sizeof(Real) == 4, bs);
-    }
-    mark(1, bs);
-    mark(4, fs);
-    if (pl) {
-      const cudaEvent_t begun = d.aux && pl->n_frame <= kFrameFirst ? d.begun : nullptr;
-      if constexpr (DEV) {
-        if (pl->n_frame) {
-          const int* tab = pl->frame_tab;
-          launch_begun(kb_pml_fused<S>, pl->n_frame, 256, pl->frame_smem, fs, begun,
-                       reinterpret_cast<const MemberDev<float>*>(pm), tab);
-        }
-      }
-      launch_frame1(*pl, pm, fs, begun);
-      if (begun) cudaStreamWaitEvent(d.st, begun, 0);
-      mark(5, fs);
-      auto band_b = [&]() {
-        mark(8, bs);
-        launch_band(*pl, pm, bs);
-        mark(9, bs);
-      };
-      if (link) {
-        band_b();
-        if (fs != bs) {
-          cudaEventRecord(d.join, bs);
-          cudaStreamWaitEvent(fs, d.join, 0);
-        }
-      }
-      mark(6, fs);
-      launch_frame2(*pl, pm, fs);
-      mark(7, fs);
-      if (!link) band_b();
-    }
-    bool fused = false;
-    if constexpr (DEV) {
-      if (!pl && has_pml(g) && !link) {
-        // FP32: single-pass frame (tile + halo in shared memory)
-        const FrameTiles ft = make_frame_tiles(g, 256);
-        const size_t smem = pml_fused_smem<S>(ft);
-        k_pml_fused<S, STREAM><<<frame_tile_count(ft), 256, smem, fs>>>(
-            g, c, ft, A, B, static_cast<const float*>(d.Sold), static_cast<float*>(d.Snew),
-            d.Uedge_out, d.bc.bc == 2 ? 1 : 0, d.flag, d.Sedge_out, src_mask);
-        fused = true;
-      }
-    }
-    if (!fused && !pl)
-      k_frame1<S, Real, DEV, STREAM><<<(g.frame_n + 127) / 128, 128, 0, fs>>>(
-          g, c, A, B, static_cast<Real*>(d.Sold), static_cast<Real*>(d.Snew), d.Uedge_out,
-          d.bc.bc == 2 ? 1 : 0, d.flag, d.Sedge_out, src_mask);
-    if (!pl) mark(5, fs);
-    auto band = [&]() {
-      mark(8, bs);
-      k_gamma<S, Real, DEV, STREAM><<<(g.ngamma + 127) / 128, 128, 0, bs>>>(
-          g, c, d.bc, A, B, d.Vtgt, link ? static_cast<Real*>(d.Sold) : nullptr,
-          link ? static_cast<Real*>(d.Snew) : nullptr);
-      mark(9, bs);
-    };
-    if (!pl) {
-      if (link) {
-        band();
-        if (fs != bs) {
-          cudaEventRecord(d.join, bs);
-          cudaStreamWaitEvent(fs, d.join, 0);
-        }
-      }
-      mark(6, fs);
-      if (has_pml(g) && !fused)
-        k_frame2<S, Real><<<(g.frame_n + 127) / 128, 128, 0, fs>>>(
-            g, c, B, static_cast<const Real*>(d.Sold), d.Sedge_out, src_mask);
-      mark(7, fs);
-      if (!link) band();
-    }
-    const int nbx = (g.Lx - g.Fe - (g.Fw / 32) * 32 + 31) / 32;
-    const int ny_in = g.Ly - g.Fs - g.Fn;
-    constexpr int BY = 4;
-    mark(2, d.st);
-    if (nbx > 0 && ny_in > 0) {
-      dim3 grid(nbx, (ny_in + BY - 1) / BY);
-      k_bulk<S, Real, DEV, STREAM><<<grid, dim3(32, BY), 0, d.st>>>(g, c, A, B, d.flag);
-    }
-    mark(3, d.st);
+    const cudaStream_t bs = d.aux ? d.aux : d.st;
+    return {bs, d.aux2 ? d.aux2 : bs};
+  }
+  static void join_streams(const Dev& d) {
     if (d.aux) {
       cudaEventRecord(d.join, d.aux);
       cudaStreamWaitEvent(d.st, d.join, 0);
@@ -528,9 +426,121 @@ struct Ops {
         cudaStreamWaitEvent(d.st, d.join2, 0);
       }
     }
-    if (pl) {
-      if (pl->n_wrap) kb_wrap_y<Real><<<dim3(pl->n_wrap, S::Q), 256, 0, d.st>>>(pm, pl->wrap_tab);
-    } else if (g.py) {
+  }
+  // Link mode: phase 2 of the frame reads the boundary nodes' new accumulator, so it waits for the
+  // band.
+  static void frame_waits_for_band(const Dev& d, cudaStream_t bs, cudaStream_t fs) {
+    if (fs == bs) return;
+    cudaEventRecord(d.join, bs);
+    cudaStreamWaitEvent(fs, d.join, 0);
+  }
+  template <bool STREAM>
+  static void launch_bulk(const Dev& d) {
+    const Geom& g = d.g;
+    const int nbx = (g.Lx - g.Fe - (g.Fw / 32) * 32 + 31) / 32;
+    const int ny_in = g.Ly - g.Fs - g.Fn;
+    constexpr int BY = 4;
+    if (nbx <= 0 || ny_in <= 0) return;
+    dim3 grid(nbx, (ny_in + BY - 1) / BY);
+    k_bulk<S, Real, DEV, STREAM><<<grid, dim3(32, BY), 0, d.st>>>(
+        g, consts(d), static_cast<const Real*>(d.A), static_cast<Real*>(d.B), d.flag);
+  }
+
+  // One step of a context: characteristic targets then boundary band, the PML frame, and the
+  // interior. The boundary-side classes run through the table-driven kernels of its one-member plan
+  // (the kernels a batch runs), so that a context computes bit for bit the same alone and in any
+  // batch; the interior kernel is the same either way.
+  static cudaError_t step_stream(const Dev& d) {
+    const bool link = d.g.link && has_pml(d.g);
+    const BatchPlan& pl = *d.plan;
+    const MemberDev<Real>* pm = static_cast<const MemberDev<Real>*>(pl.desc[d.which]);
+    auto mark = [&](int k, cudaStream_t s) {
+      if (d.ev) cudaEventRecord(d.ev[k], s);
+    };
+    const auto [bs, fs] = fork_streams(d);
+    mark(0, bs);
+    {
+      const cudaEvent_t begun = d.aux ? d.begun : nullptr;
+      launch_nrbc_batch(pl.tgt[d.which], pl.tgt_tab, pl.n_tgt, sizeof(Real) == 4, pl.tgt_threads,
+                        pl.tgt_smem, bs, begun);
+      if (begun && fs != bs && pl.n_tgt) cudaStreamWaitEvent(fs, begun, 0);
+    }
+    mark(1, bs);
+    mark(4, fs);
+    const cudaEvent_t begun = d.aux && pl.n_frame <= kFrameFirst ? d.begun : nullptr;
+    if constexpr (DEV) {
+      if (pl.n_frame) {
+        const int* tab = pl.frame_tab;
+        launch_begun(kb_pml_fused<S>, pl.n_frame, 256, pl.frame_smem, fs, begun, pm, tab);
+      }
+    }
+    launch_frame1(pl, pm, fs, begun);
+    if (begun) cudaStreamWaitEvent(d.st, begun, 0);
+    mark(5, fs);
+    auto band = [&, bs = bs]() {
+      mark(8, bs);
+      launch_band(pl, pm, bs);
+      mark(9, bs);
+    };
+    if (link) {
+      band();
+      frame_waits_for_band(d, bs, fs);
+    }
+    mark(6, fs);
+    launch_frame2(pl, pm, fs);
+    mark(7, fs);
+    if (!link) band();
+    mark(2, d.st);
+    launch_bulk<true>(d);
+    mark(3, d.st);
+    join_streams(d);
+    if (pl.n_wrap) kb_wrap_y<Real><<<dim3(pl.n_wrap, S::Q), 256, 0, d.st>>>(pm, pl.wrap_tab);
+    return cudaGetLastError();
+  }
+
+  // The collision of the initial state: populations read in place, the boundary targets as they
+  // were set.
+  static cudaError_t step_initial(const Dev& d) {
+    const Geom& g = d.g;
+    const Consts<Real>& c = consts(d);
+    const Real* A = static_cast<const Real*>(d.A);
+    Real* B = static_cast<Real*>(d.B);
+    const bool link = g.link && has_pml(g);
+    // Appendix PML source terms: only with a characteristic BC and a PML
+    const int src_mask = (d.bc.bc == 2 && has_pml(g)) ? (d.bc.pml_source & 7) : 0;
+    const auto [bs, fs] = fork_streams(d);
+    bool fused = false;
+    if constexpr (DEV) {
+      if (has_pml(g) && !link) {
+        // FP32: single-pass frame (tile + halo in shared memory)
+        const FrameTiles ft = make_frame_tiles(g, 256);
+        const size_t smem = pml_fused_smem<S>(ft);
+        k_pml_fused<S><<<frame_tile_count(ft), 256, smem, fs>>>(
+            g, c, ft, A, B, static_cast<const float*>(d.Sold), static_cast<float*>(d.Snew),
+            d.Uedge_out, d.bc.bc == 2 ? 1 : 0, d.flag, d.Sedge_out, src_mask);
+        fused = true;
+      }
+    }
+    if (!fused)
+      k_frame1<S, Real, DEV><<<(g.frame_n + 127) / 128, 128, 0, fs>>>(
+          g, c, A, B, static_cast<Real*>(d.Sold), static_cast<Real*>(d.Snew), d.Uedge_out,
+          d.bc.bc == 2 ? 1 : 0, d.flag, d.Sedge_out, src_mask);
+    auto band = [&, bs = bs]() {
+      k_gamma<S, Real, DEV><<<(g.ngamma + 127) / 128, 128, 0, bs>>>(
+          g, c, d.bc, A, B, d.Vtgt, link ? static_cast<Real*>(d.Sold) : nullptr,
+          link ? static_cast<Real*>(d.Snew) : nullptr);
+    };
+    if (link) {
+      band();
+      frame_waits_for_band(d, bs, fs);
+    }
+    if (has_pml(g) && !fused)
+      k_frame2<S, Real><<<(g.frame_n + 127) / 128, 128, 0, fs>>>(
+          g, c, B, static_cast<const Real*>(d.Sold), d.Sedge_out, src_mask);
+    if (!link) band();
+    launch_bulk<false>(d);
+    join_streams(d);
+    if (g.py) {
       const long long n = (long long)(g.Lx + 2 * g.M) * g.M;
       k_wrap_y<Real><<<dim3(unsigned((n + 255) / 256), S::Q), 256, 0, d.st>>>(g, B);
     }
@@ -538,7 +548,7 @@ struct Ops {
   }
 
   static cudaError_t step(const Dev& d, bool stream) {
-    return stream ? step_impl<true>(d) : step_impl<false>(d);
+    return stream ? step_stream(d) : step_initial(d);
   }
 
   static cudaError_t init_eq(const Dev& d, const double* rho, const double* ux, const double* uy,
@@ -607,11 +617,8 @@ struct Ops {
       return cudaFuncSetAttribute(kb_bulk<S, Real, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)sizeof(double) * node_smem<S, Real>(256));
     if constexpr (DEV) {
-      cudaError_t e = cudaFuncSetAttribute(k_pml_fused<S, true>,
+      cudaError_t e = cudaFuncSetAttribute(k_pml_fused<S>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_pml_fused<S, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kb_pml_fused<S>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);

@@ -229,7 +229,8 @@ __device__ __forceinline__ void pml_fused_tile(const Geom& g, const Consts<float
   }
 }
 
-template <class S, bool STREAM>
+// The initial state's frame (streaming steps: kb_pml_fused).
+template <class S>
 __global__ void __launch_bounds__(256) k_pml_fused(Geom g, Consts<float> c, FrameTiles ft,
                                                    const float* __restrict__ A,
                                                    float* __restrict__ B,
@@ -238,8 +239,8 @@ __global__ void __launch_bounds__(256) k_pml_fused(Geom g, Consts<float> c, Fram
                                                    int save_edges, int* flag, double* Sedge,
                                                    int src_mask) {
   extern __shared__ float smem[];
-  pml_fused_tile<S, STREAM>(g, c, ft, A, B, Sold, Snew, Uedge, save_edges, flag, Sedge, src_mask,
-                            blockIdx.x, smem);
+  pml_fused_tile<S, false>(g, c, ft, A, B, Sold, Snew, Uedge, save_edges, flag, Sedge, src_mask,
+                           blockIdx.x, smem);
 }
 
 }  // namespace lbm
