@@ -164,7 +164,7 @@ int halo_of(int q) { return q == 9 ? 1 : 3; }
 // Fixed-point constants of an FP64 context (fixed.cuh), from the doubles that the FP64 arithmetic
 // multiplies by: the sums of these miss the quadrature by 1e-16, so T drifts by 3e-16 a step, and
 // both arithmetics then drift alike. They stay off where that arithmetic does
-// not apply: omega outside (0, 2), or a mean state outside its range.
+// not apply: omega outside (0, 2), a mean density beyond 2^60 or a mean equilibrium beyond 2^59 units.
 template <class S>
 void fixed_consts(const double* w, double r2, double omega, const lbm_bc_params& bp,
                   const double* fbar, fx::Consts& c) {
@@ -292,6 +292,19 @@ static void free_all(lbm_ctx* ctx) {
   if (ctx->hflag) cudaFreeHost(ctx->hflag);
 }
 
+// Whether a context whose initial state has `outside` nodes out of the fixed-point range updates
+// its nodes in fixed point. A node that turns out to be outside costs the attempt and then the FP64
+// update with the fixed-point kernel's registers, so a state that is outside (almost) everywhere
+// takes kernels of its own. us a step, periodic, fixed point with fallback / all FP64: D2Q37 1024^2
+// 743 / 754 with 90 % outside, 784 / 754 with 97 %, 791 / 754 with all; D2Q17 381 / 394, 401 / 394,
+// 404 / 394; 300^2 with a PML 20 wide (D2Q37) 146 / 147, 147 / 147, 155 / 147; D2Q37 128^2 with all
+// 47 / 22 (an idle chip: the four-warp kernels' blocks share SMs with the interior's). That last
+// kind, small and without a PML, also loses with a fifth or more outside (25 / 22 at 25 %).
+static bool fixed_form(const lbm_ctx* ctx, int outside) {
+  if (ctx->prec != LBM_FP64 || !ctx->dev.cd.fx.on) return false;
+  return 16ll * outside <= 15ll * ctx->g.Lx * ctx->g.Ly;
+}
+
 // Steps in the longer of a context's (and a batch's) two graphs: even, so that a replay starts and
 // ends with the same buffer parity. Between two graphs of one step the device idles for a fork, a
 // join and a launch, inside one graph for dependent nodes only: a 512^2 FP32 step 66 -> 52 us, a
@@ -319,6 +332,17 @@ static void set_roles(lbm_ctx* ctx, int a, int s) {
   d.Uedge_out = ctx->Uedge + (1 - a) * edge_slots(ctx->g);
   d.Sedge_in = ctx->Sedge + a * source_slots(ctx->g);
   d.Sedge_out = ctx->Sedge + (1 - a) * source_slots(ctx->g);
+}
+
+// An FP64 context's form of the node update (BatchPlan::fixed); no step may be in flight.
+static void set_form(lbm_ctx* ctx, bool fixed) {
+  if (fixed == ctx->dev.fixed) return;
+  ctx->dev.fixed = ctx->plan.fixed = fixed;
+  for (int k = 0; k < 2; ++k) {
+    if (ctx->graph[k]) cudaGraphExecDestroy(ctx->graph[k]);
+    if (ctx->many[k]) cudaGraphExecDestroy(ctx->many[k]);
+    ctx->graph[k] = ctx->many[k] = nullptr;
+  }
 }
 
 static lbm_status check_ready(lbm_ctx* ctx) {
@@ -598,6 +622,7 @@ lbm_status lbm_create(const lbm_grid* grid, lbm_stencil stencil, double tau, int
   if (q == 37) fixed_consts<D2Q37>(ctx->w, d.cd.r2, ctx->omega, bp, fbar, d.cd.fx);
   else if (q == 17) fixed_consts<D2Q17>(ctx->w, d.cd.r2, ctx->omega, bp, fbar, d.cd.fx);
   else fixed_consts<D2Q9>(ctx->w, d.cd.r2, ctx->omega, bp, fbar, d.cd.fx);
+  d.fixed = precision == LBM_FP64 && d.cd.fx.on;
   d.cf.r = (float)ctx->r; d.cf.r2 = (float)(ctx->r * ctx->r); d.cf.omega = (float)ctx->omega;
   d.cf.sigma_max = (float)sg.sigma_max; d.cf.power = sg.power; d.cf.split = sg.split;
   {
@@ -720,7 +745,10 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* rho, const double* ux, const dou
   *ctx->hflag = 0;
   Dev& d = ctx->dev;
   set_roles(ctx, 0, 0);
-  LBM_CK(ctx->ops.init_eq(d, src[0], src[1], src[2], src[3]));
+  int* outside = reinterpret_cast<int*>(ctx->dout + 15);   // past the reductions' twelve values
+  LBM_CK(cudaMemsetAsync(outside, 0, sizeof(int), ctx->st));
+  LBM_CK(ctx->ops.init_eq(d, src[0], src[1], src[2], src[3], outside));
+  LBM_CK(cudaMemcpyAsync(ctx->hout + 15, outside, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
   if (ctx->bc == LBM_BC_NRBC) {
     k_init_targets<<<(g.nb + 127) / 128, 128, 0, ctx->st>>>(g, src[0], src[1], src[2], src[3],
                                                             d.Vtgt);
@@ -729,6 +757,7 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* rho, const double* ux, const dou
   // initial collision (no streaming): buffer 0 holds f^0, buffer 1 receives f*^0
   LBM_CK(ctx->ops.step(d, false));
   LBM_CK(cudaStreamSynchronize(ctx->st));
+  set_form(ctx, fixed_form(ctx, *reinterpret_cast<const int*>(ctx->hout + 15)));
   ctx->cur = 1;
   ctx->scur = 1;
   ctx->steps = 0;
@@ -1041,7 +1070,8 @@ lbm_status lbm_checkpoint(lbm_ctx* ctx, void* host, size_t bytes) {
   CkptHeader h{kMagic, ctx->q, ctx->g.nx, ctx->g.ny, pack_widths(ctx), (int64_t)ctx->prec,
                ctx->steps,
                (int64_t)(ctx->prev_valid ? 1 : 0) | (int64_t)(ctx->prev_prestream ? 2 : 0) |
-                   ((int64_t)ctx->g.py << 2) | ((int64_t)ctx->g.link << 3)};
+                   ((int64_t)ctx->g.py << 2) | ((int64_t)ctx->g.link << 3) |
+                   (int64_t)(ctx->dev.fixed != (ctx->prec == LBM_FP64 && ctx->dev.cd.fx.on) ? 16 : 0)};
   std::memcpy(p, &h, sizeof h);
   p += sizeof h;
   const cudaMemcpyKind k = cudaMemcpyDeviceToHost;
@@ -1092,6 +1122,7 @@ lbm_status lbm_restore(lbm_ctx* ctx, const void* host, size_t bytes) {
   ctx->steps = h.steps;
   ctx->prev_valid = (h.flags & 1) != 0;
   ctx->prev_prestream = (h.flags & 2) != 0;
+  set_form(ctx, ctx->prec == LBM_FP64 && ctx->dev.cd.fx.on && !(h.flags & 16));
   ctx->initialized = true;
   *ctx->hflag = 0;
   return LBM_OK;
@@ -1101,7 +1132,7 @@ lbm_status lbm_restore(lbm_ctx* ctx, const void* host, size_t bytes) {
 
 // --------------------------------------------------------------------------------------------
 // Batched execution (see lbm.h): the members are grouped by (stencil, precision, PML gradient
-// mode); each group is one plan whose kernels each cover every member of the group in one
+// mode, FP64 form); each group is one plan whose kernels each cover every member of the group in one
 // launch (a table of (member, tile) entries), and one step of all groups is one captured graph
 // per buffer-parity state.
 #include <map>
@@ -1130,7 +1161,8 @@ struct lbm_batch {
   cudaEvent_t fork = nullptr, join = nullptr, join2 = nullptr, begun = nullptr;
   int device = -1;
   std::vector<lbm_ctx*> members;
-  std::vector<int> base;                  // members' buffer parity when the plans were built
+  std::vector<int> base;                  // members' buffer parity and FP64 form (Dev::fixed)
+  std::vector<char> form;                 // when the plans were built
   std::vector<BatchGroup> groups;
   cudaGraphExec_t graph[2] = {nullptr, nullptr}, many[2] = {nullptr, nullptr};
   int tx = 0, by = 0;                     // bulk tile shape; 0: from the tuning cache / default
@@ -1194,10 +1226,10 @@ static lbm_status batch_build(lbm_batch* b) {
     tx = it != g_tune_cache.end() ? it->second.first : 32;
     by = it != g_tune_cache.end() ? it->second.second : 4;
   }
-  std::map<std::tuple<int, int, int>, int> gi;
+  std::map<std::tuple<int, int, int, int>, int> gi;
   for (int m = 0; m < (int)b->members.size(); ++m) {
     lbm_ctx* c = b->members[m];
-    auto key = std::make_tuple(c->q, (int)c->prec, c->g.link);
+    auto key = std::make_tuple(c->q, (int)c->prec, c->g.link, (int)c->dev.fixed);
     auto it = gi.find(key);
     if (it == gi.end()) {
       gi[key] = (int)b->groups.size();
@@ -1207,11 +1239,13 @@ static lbm_status batch_build(lbm_batch* b) {
     }
   }
   b->base.resize(b->members.size());
+  b->form.resize(b->members.size());
   for (auto& G : b->groups) {
     std::vector<Dev> d0, d1;
     for (int m : G.idx) {
       lbm_ctx* c = b->members[m];
       b->base[m] = c->cur;
+      b->form[m] = c->dev.fixed;
       set_roles(c, c->cur, c->scur);
       d0.push_back(c->dev);
       set_roles(c, c->cur ^ 1, c->scur ^ 1);
@@ -1292,13 +1326,13 @@ lbm_status lbm_batch_step(lbm_batch* b, int n) {
   LBM_CK(cudaSetDevice(b->device));
   for (int k = 0; k < n; ++k) {
     // parity state of the members against the plans (a member stepped on its own since
-    // then makes the states disagree: rebuild)
+    // then makes the states disagree, one initialized again may have another form: rebuild)
     int state = -1;
     if (b->built) {
       for (size_t m = 0; m < b->members.size(); ++m) {
         const int s = b->members[m]->cur != b->base[m] ? 1 : 0;
         if (state < 0) state = s;
-        else if (s != state) { state = -2; break; }
+        if (s != state || b->form[m] != (char)b->members[m]->dev.fixed) { state = -2; break; }
       }
     }
     if (!b->built || state < 0) {

@@ -545,5 +545,16 @@ LBM_HD bool state(const Moments& m, const Consts& c, State& u) {
   return in_range(u);
 }
 
+// The state of given density, r u and temperature; false out of the range.
+LBM_HD bool state_of(double rho, double X, double Y, double T, const Consts& c, State& u) {
+  const double p = rho * pow2(-c.E), th = T - 1.0;
+  if (!(p < 2.0 && p > 0.5 && fabs(X) < 2.0 && fabs(Y) < 2.0 && fabs(th) < 2.0)) return false;
+  u.rho = fixed60(p) >> 2;
+  u.X = fixed60(X);
+  u.Y = fixed60(Y);
+  u.th = fixed60(th);
+  return in_range(u);
+}
+
 }  // namespace fx
 }  // namespace lbm

@@ -536,13 +536,14 @@ __device__ __noinline__ void bulk_outside(const Geom& g, const Consts<double>& c
   bulk_plain<S, double, false, STREAM>(g, c, A, B, flag, idx);
 }
 
-template <class S, class Real, bool DEV, bool STREAM>
+// FIXED (FP64 kernels only): in fixed point where the node's state allows it.
+template <class S, class Real, bool DEV, bool STREAM, bool FIXED>
 __device__ __forceinline__ void bulk_node(const Geom& g, const Consts<Real>& c,
                                           const Real* __restrict__ A, Real* __restrict__ B,
                                           int* flag, int x, int y, double* f, int stride) {
   if (x < g.Fw || x >= g.Lx - g.Fe || y >= g.Ly - g.Fn) return;
   const long long idx = gindex(g, x, y);
-  if constexpr (sizeof(Real) == 8) {
+  if constexpr (FIXED) {
     if (c.fx.on && bgk_fixed<S, STREAM>(g, c.fx, A, B, idx, f, stride)) return;
     bulk_outside<S, STREAM>(g, c, A, B, flag, idx);
   } else {
@@ -550,27 +551,27 @@ __device__ __forceinline__ void bulk_node(const Geom& g, const Consts<Real>& c,
   }
 }
 
-// Blocks of 128 threads per SM of the FP64 interior. The update is bound by integer issue (about
+// Blocks of 128 threads per SM of the fixed-point interior. The update is bound by integer issue (about
 // 4500 instructions per D2Q37 node), so more warps help little. Measured at 1024^2, blocks per SM:
 // D2Q37 3 236 us (before the out-of-line FP64 form), 4 202, 5 199 (all its shared memory allows);
 // D2Q17 5 120, 6 95, 8 95, 10 97; D2Q9 8 53, 10 54. In FP64 arithmetic 738, 385 and 203 us.
-template <class S, class Real>
+template <class S, bool FIXED>
 constexpr int bulk_blocks() {
-  return sizeof(Real) == 4 ? 0 : S::Q == 37 ? 5 : S::Q == 17 ? 6 : 8;   // 0: no bound
+  return !FIXED ? 0 : S::Q == 37 ? 5 : S::Q == 17 ? 6 : 8;   // 0: no bound
 }
-// Shared memory of an FP64 block of n threads: one value per direction and thread.
-template <class S, class Real>
+// Shared memory of a fixed-point block of n threads: one value per direction and thread.
+template <class S, bool FIXED>
 __host__ __device__ constexpr int node_smem(int n) {
-  return sizeof(Real) == 8 ? S::Q * n : 1;
+  return FIXED ? S::Q * n : 1;
 }
 
-template <class S, class Real, bool DEV, bool STREAM>
-__global__ void __launch_bounds__(sizeof(Real) == 8 ? 128 : 256, bulk_blocks<S, Real>()) k_bulk(
+template <class S, class Real, bool DEV, bool STREAM, bool FIXED>
+__global__ void __launch_bounds__(FIXED ? 128 : 256, bulk_blocks<S, FIXED>()) k_bulk(
     const __grid_constant__ Geom g, const __grid_constant__ Consts<Real> c,
     const Real* __restrict__ A, Real* __restrict__ B, int* flag) {
-  __shared__ double f[node_smem<S, Real>(128)];
+  __shared__ double f[node_smem<S, FIXED>(128)];
   const int x0 = (g.Fw / 32) * 32;
-  bulk_node<S, Real, DEV, STREAM>(g, c, A, B, flag, x0 + blockIdx.x * 32 + threadIdx.x,
+  bulk_node<S, Real, DEV, STREAM, FIXED>(g, c, A, B, flag, x0 + blockIdx.x * 32 + threadIdx.x,
                                   g.Fs + blockIdx.y * blockDim.y + threadIdx.y,
                                   f + threadIdx.y * 32 + threadIdx.x, 128);
 }
@@ -802,7 +803,7 @@ __device__ __noinline__ void frame1_outside(const Geom& g, const Consts<double>&
                                          src_mask, fi, x, y, nullptr);
 }
 
-template <class S, class Real, bool DEV, bool STREAM, bool STAGE = false>
+template <class S, class Real, bool DEV, bool STREAM, bool FIXED, bool STAGE = false>
 __device__ __forceinline__ void frame1_node(const Geom& g, const Consts<Real>& c,
                                             const Real* __restrict__ A, Real* __restrict__ B,
                                             Real* __restrict__ Sold,
@@ -813,7 +814,7 @@ __device__ __forceinline__ void frame1_node(const Geom& g, const Consts<Real>& c
   if (fi >= g.frame_n) return;
   int x, y;
   frame_xy(g, fi, x, y);
-  if constexpr (sizeof(Real) == 8) {
+  if constexpr (FIXED) {
     if (c.fx.on && frame1_fixed<S, STREAM>(g, c, A, B, Sold, Snew, Uedge, save_edges, Sedge,
                                            src_mask, fi, x, y, stage, stride))
       return;
@@ -854,22 +855,22 @@ __device__ __forceinline__ void frame1_split(const Geom& g, const Consts<double>
   }
 }
 
-// Blocks of 128 threads per SM of the FP64 frame and band kernels. Measured on the 1024^2 frame,
+// Blocks of 128 threads per SM of the fixed-point frame and band kernels. Measured on the 1024^2 frame,
 // phase 1: D2Q37 3 116 us, 4 107, 5 (spills) 124; in FP64 arithmetic 275 us.
-template <class S, class Real>
+template <class S, bool FIXED>
 constexpr int edge_blocks() {
-  return sizeof(Real) == 4 ? 0 : S::Q == 37 ? 4 : S::Q == 17 ? 5 : 8;
+  return !FIXED ? 0 : S::Q == 37 ? 4 : S::Q == 17 ? 5 : 8;
 }
 
 // The initial state's frame (streaming steps: kb_frame1).
 template <class S, class Real, bool DEV>
-__global__ void __launch_bounds__(128, edge_blocks<S, Real>()) k_frame1(
+__global__ void __launch_bounds__(128, edge_blocks<S, !DEV>()) k_frame1(
     const __grid_constant__ Geom g, const __grid_constant__ Consts<Real> c,
     const Real* __restrict__ A, Real* __restrict__ B, Real* __restrict__ Sold,
     Real* __restrict__ Snew, double* Uedge, int save_edges, int* flag, double* Sedge,
     int src_mask) {
-  __shared__ double f[node_smem<S, Real>(128)];
-  frame1_node<S, Real, DEV, false>(g, c, A, B, Sold, Snew, Uedge, save_edges, flag, Sedge,
+  __shared__ double f[node_smem<S, !DEV>(128)];
+  frame1_node<S, Real, DEV, false, !DEV>(g, c, A, B, Sold, Snew, Uedge, save_edges, flag, Sedge,
                                    src_mask, blockIdx.x * blockDim.x + threadIdx.x,
                                    reinterpret_cast<Real*>(f) + threadIdx.x, 128);
 }
@@ -1095,14 +1096,8 @@ __device__ inline int q_slot(const Geom& g, int x, int y) {
 __device__ __forceinline__ bool target_state(const Geom& g, const fx::Consts& c, const BcParams& bc,
                                              const double* __restrict__ Vtgt, int b,
                                              fx::State& ut) {
-  const double X = bc.r * Vtgt[g.nb + b], Y = bc.r * Vtgt[2 * g.nb + b];
-  const double rho = Vtgt[b] * fx::pow2(-c.E), th = Vtgt[3 * g.nb + b] - 1.0;
-  if (!(rho < 2.0 && rho > 0.5 && fabs(X) < 2.0 && fabs(Y) < 2.0 && fabs(th) < 2.0)) return false;
-  ut.rho = fx::fixed60(rho) >> 2;
-  ut.X = fx::fixed60(X);
-  ut.Y = fx::fixed60(Y);
-  ut.th = fx::fixed60(th);
-  return fx::in_range(ut);
+  return fx::state_of(Vtgt[b], bc.r * Vtgt[g.nb + b], bc.r * Vtgt[2 * g.nb + b],
+                      Vtgt[3 * g.nb + b], c, ut);
 }
 
 // The same for an FP64 node in fixed point from the fluid node's state u and integers and, on an
@@ -1252,7 +1247,7 @@ __device__ __forceinline__ bool gamma_place(const Geom& g, const BcParams& bc, i
   return true;
 }
 
-template <class S, class Real, bool DEV, bool STREAM>
+template <class S, class Real, bool DEV, bool STREAM, bool FIXED>
 __device__ __forceinline__ void gamma_node(const Geom& g, const Consts<Real>& c,
                                            const BcParams& bc, const Real* __restrict__ A,
                                            Real* __restrict__ B,
@@ -1264,7 +1259,7 @@ __device__ __forceinline__ void gamma_node(const Geom& g, const Consts<Real>& c,
   long long src, dst;
   int b;
   if (!gamma_place(g, bc, t, src, dst, b)) return;
-  if constexpr (sizeof(Real) == 8) {
+  if constexpr (FIXED) {
     fx::State u, ut;
     if (c.fx.on && (b < 0 || target_state(g, c.fx, bc, Vtgt, b, ut)) &&
         pull_fixed<S, STREAM>(f, stride, A, g, c.fx, src, u))
@@ -1299,13 +1294,14 @@ __device__ __forceinline__ void gamma_split(const Geom& g, const Consts<double>&
 
 // The initial state's band (streaming steps: kb_gamma).
 template <class S, class Real, bool DEV>
-__global__ void __launch_bounds__(128, edge_blocks<S, Real>()) k_gamma(
+__global__ void __launch_bounds__(128, edge_blocks<S, !DEV>()) k_gamma(
     const __grid_constant__ Geom g, const __grid_constant__ Consts<Real> c,
     const __grid_constant__ BcParams bc, const Real* __restrict__ A, Real* __restrict__ B,
     const double* __restrict__ Vtgt, Real* __restrict__ Sold, Real* __restrict__ Snew) {
-  __shared__ double f[node_smem<S, Real>(128)];
-  gamma_node<S, Real, DEV, false>(g, c, bc, A, B, Vtgt, Sold, Snew,
-                                  blockIdx.x * blockDim.x + threadIdx.x, f + threadIdx.x, 128);
+  __shared__ double f[node_smem<S, !DEV>(128)];
+  gamma_node<S, Real, DEV, false, !DEV>(g, c, bc, A, B, Vtgt, Sold, Snew,
+                                        blockIdx.x * blockDim.x + threadIdx.x, f + threadIdx.x,
+                                        128);
 }
 
 // Periodic y axis: the M rows below y = 0 and above y = Ly - 1 (boundary columns included)

@@ -46,6 +46,7 @@ struct Dev {
   // parity of this launch; streaming steps run the boundary-side classes through it
   const struct BatchPlan* plan;
   int which;
+  bool fixed;        // FP64: nodes are updated in fixed point (BatchPlan::fixed)
 };
 
 constexpr int kKernelClasses = 5;
@@ -60,7 +61,8 @@ struct TgtDesc {
   double* V;
 };
 
-// Work list of a batch of instances with the same stencil, precision and PML gradient mode:
+// Work list of a batch of instances with the same stencil, precision, PML gradient mode and FP64
+// form:
 // one launch per kernel class over a table of (member, tile / block) entries that spans all
 // instances (see lbm_batch_step). The member descriptors exist for the two buffer-parity
 // states the batch alternates between; everything lives in one device allocation.
@@ -80,6 +82,8 @@ struct BatchPlan {
   int tgt_threads = 0, q = 0;
   int tx = 32, by = 4;        // bulk tile shape (blockDim)
   bool link = false;
+  bool fixed = false;         // FP64 nodes in fixed point, except those out of its range; else all
+                              // in FP64, by kernels of their own (more registers, no attempt first)
   bool split = false;         // small launches may run four warps on 32 nodes (FP64)
   void* mem = nullptr;
 };
@@ -88,7 +92,9 @@ struct OpsTable {
   cudaError_t (*prepare)(const double* w);   // kernel attributes and the quadrature weights
                                              // (constant memory) on the current device
   cudaError_t (*step)(const Dev&, bool stream);
-  cudaError_t (*init_eq)(const Dev&, const double*, const double*, const double*, const double*);
+  // outside: adds the nodes out of the range of the fixed-point update (FP64)
+  cudaError_t (*init_eq)(const Dev&, const double*, const double*, const double*, const double*,
+                         int* outside);
   cudaError_t (*fields)(const Dev&, const void* src, bool stream, int region, double* const o[4],
                         const double* const r[4], int mode, double* partials, int* nblocks);
   cudaError_t (*export_pop)(const Dev&, const void* src, double* out);

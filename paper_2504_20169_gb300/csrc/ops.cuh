@@ -16,11 +16,13 @@
 namespace lbm {
 
 // f^0 = f_eq(rho, u, T) on F (Sec. 2 initialization) and, on P and its ring, the accumulator
-// S^(-1) = -f_hat^0 / 2 so that Q^0 = S^(-1) + f_hat^0 / 2 = 0.
+// S^(-1) = -f_hat^0 / 2 so that Q^0 = S^(-1) + f_hat^0 / 2 = 0. FP64: *outside counts the nodes out
+// of the range of the fixed-point update.
 template <class S, class Real, bool DEV>
 __global__ void k_init_eq(Geom g, Consts<Real> c, const double* __restrict__ rho,
                           const double* __restrict__ ux, const double* __restrict__ uy,
-                          const double* __restrict__ T, Real* __restrict__ A, Real* __restrict__ Sold) {
+                          const double* __restrict__ T, Real* __restrict__ A, Real* __restrict__ Sold,
+                          int* outside) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y;
   if (x >= g.Lx) return;
@@ -38,11 +40,20 @@ __global__ void k_init_eq(Geom g, Consts<Real> c, const double* __restrict__ rho
   const long long idx = gindex(g, x, y);
   const bool has_q = pml_node<Real>(g, x, y).has_q;
   const int fi = has_q ? frame_index(g, x, y) : 0;
+  int low = 1 << 20;
 #pragma unroll
   for (int i = 0; i < S::Q; ++i) {
     const Real eq = eq_dir<S, Real, DEV>(i, m, kc, c);
     A[(long long)i * g.plane + idx] = eq;
     if (has_q) Sold[(long long)i * g.Sp + fi] = Real(-0.5) * (eq - c.eqbar[i]);
+    if constexpr (!DEV) fx::load(eq, c.fx.shell[fx::shell_position<S>(i)].fe, c.fx.E, low);
+  }
+  if constexpr (!DEV) {
+    // nodes that the fixed-point update would hand to the FP64 one
+    fx::State u;
+    const bool out = low < 3 || !fx::state_of(r0, c.r * vx, c.r * vy, T0, c.fx, u);
+    const unsigned act = __activemask(), all = __ballot_sync(act, out);
+    if (all && (threadIdx.x & 31) == __ffs(act) - 1) atomicAdd(outside, __popc(all));
   }
 }
 
@@ -222,15 +233,15 @@ struct MemberDev {
   int src_mask;
 };
 
-template <class S, class Real, bool DEV>
-__global__ void __launch_bounds__(256, bulk_blocks<S, Real>() / 2) kb_bulk(const MemberDev<Real>* __restrict__ mem,
-                                               const int* __restrict__ tab) {
-  extern __shared__ double bsh[];   // FP64: the nodes of the block (node_smem values)
+template <class S, class Real, bool DEV, bool FIXED>
+__global__ void __launch_bounds__(256, bulk_blocks<S, FIXED>() / 2) kb_bulk(
+    const MemberDev<Real>* __restrict__ mem, const int* __restrict__ tab) {
+  extern __shared__ double bsh[];   // fixed point: the nodes of the block (node_smem values)
   const int* e = tab + 3 * blockIdx.x;
   const MemberDev<Real>& md = mem[e[0]];
   const Geom g = md.g;
   const int x0 = (g.Fw / 32) * 32;
-  bulk_node<S, Real, DEV, true>(g, md.c, md.A, md.B, md.flag,
+  bulk_node<S, Real, DEV, true, FIXED>(g, md.c, md.A, md.B, md.flag,
                                 x0 + e[1] * blockDim.x + threadIdx.x,
                                 g.Fs + e[2] * blockDim.y + threadIdx.y,
                                 bsh + threadIdx.y * blockDim.x + threadIdx.x,
@@ -247,22 +258,22 @@ __global__ void __launch_bounds__(256) kb_pml_fused(const MemberDev<float>* __re
                           md.bc.bc == 2 ? 1 : 0, md.flag, md.Sedge_out, md.src_mask, e[1], smem);
 }
 
-template <class S, class Real, bool DEV>
-__global__ void __launch_bounds__(128, edge_blocks<S, Real>()) kb_frame1(const MemberDev<Real>* __restrict__ mem,
-                                                 const int* __restrict__ tab) {
+template <class S, class Real, bool DEV, bool FIXED>
+__global__ void __launch_bounds__(128, edge_blocks<S, FIXED>()) kb_frame1(
+    const MemberDev<Real>* __restrict__ mem, const int* __restrict__ tab) {
   const int* e = tab + 2 * blockIdx.x;
   const MemberDev<Real>& md = mem[e[0]];
   const Geom g = md.g;
   if constexpr (sizeof(Real) == 4) {
     // FP32: the node's accumulator is staged in shared memory by cp.async during the pull
     __shared__ float stage[128 * S::Q];
-    frame1_node<S, Real, DEV, true, true>(g, md.c, md.A, md.B, md.Sold, md.Snew, md.Uedge_out,
+    frame1_node<S, Real, DEV, true, FIXED, true>(g, md.c, md.A, md.B, md.Sold, md.Snew, md.Uedge_out,
                                           md.bc.bc == 2 ? 1 : 0, md.flag, md.Sedge_out,
                                           md.src_mask, e[1] * blockDim.x + threadIdx.x,
                                           reinterpret_cast<Real*>(stage) + threadIdx.x * S::Q);
   } else {
-    __shared__ double f[node_smem<S, Real>(128)];
-    frame1_node<S, Real, DEV, true>(g, md.c, md.A, md.B, md.Sold, md.Snew, md.Uedge_out,
+    __shared__ double f[node_smem<S, FIXED>(128)];
+    frame1_node<S, Real, DEV, true, FIXED>(g, md.c, md.A, md.B, md.Sold, md.Snew, md.Uedge_out,
                                     md.bc.bc == 2 ? 1 : 0, md.flag, md.Sedge_out, md.src_mask,
                                     e[1] * blockDim.x + threadIdx.x, f + threadIdx.x, 128);
   }
@@ -287,21 +298,21 @@ __global__ void __launch_bounds__(128) kb_frame2(const MemberDev<Real>* __restri
   }
 }
 
-template <class S, class Real, bool DEV>
-__global__ void __launch_bounds__(128, edge_blocks<S, Real>()) kb_gamma(const MemberDev<Real>* __restrict__ mem,
-                                                const int* __restrict__ tab) {
+template <class S, class Real, bool DEV, bool FIXED>
+__global__ void __launch_bounds__(128, edge_blocks<S, FIXED>()) kb_gamma(
+    const MemberDev<Real>* __restrict__ mem, const int* __restrict__ tab) {
   const int* e = tab + 2 * blockIdx.x;
   const MemberDev<Real>& md = mem[e[0]];
   const Geom g = md.g;
   const bool link = g.link && has_pml(g);
-  __shared__ double f[node_smem<S, Real>(128)];
-  gamma_node<S, Real, DEV, true>(g, md.c, md.bc, md.A, md.B, md.Vtgt,
+  __shared__ double f[node_smem<S, FIXED>(128)];
+  gamma_node<S, Real, DEV, true, FIXED>(g, md.c, md.bc, md.A, md.B, md.Vtgt,
                                  link ? md.Sold : nullptr, link ? md.Snew : nullptr,
                                  e[1] * blockDim.x + threadIdx.x, f + threadIdx.x, 128);
 }
 
-// Small FP64 launches: four warps on 32 nodes, four blocks to an entry of the table (entries whose
-// member is out of the fixed-point arithmetic altogether have one warp do the node).
+// Small FP64 launches: four warps on 32 nodes, four blocks to an entry of the table (phase 1 and the
+// band in fixed point; a node out of its range is one warp's).
 template <class S>
 __global__ void __launch_bounds__(128) kb_frame1_split(const MemberDev<double>* __restrict__ mem,
                                                        const int* __restrict__ tab) {
@@ -377,12 +388,15 @@ struct Ops {
     if (!p.n_f1) return;
     const int* tab = p.f1_tab;
     if constexpr (!DEV) {
-      if (p.split && p.n_f1 <= kSplitBlocks) {
-        launch_begun(kb_frame1_split<S>, 4 * p.n_f1, 128, 0, s, begun, m, tab);
+      if (p.fixed) {
+        if (p.split && p.n_f1 <= kSplitBlocks)
+          launch_begun(kb_frame1_split<S>, 4 * p.n_f1, 128, 0, s, begun, m, tab);
+        else
+          launch_begun(kb_frame1<S, Real, DEV, true>, p.n_f1, 128, 0, s, begun, m, tab);
         return;
       }
     }
-    launch_begun(kb_frame1<S, Real, DEV>, p.n_f1, 128, 0, s, begun, m, tab);
+    launch_begun(kb_frame1<S, Real, DEV, false>, p.n_f1, 128, 0, s, begun, m, tab);
   }
   static void launch_frame2(const BatchPlan& p, const MemberDev<Real>* m, cudaStream_t s) {
     if (!p.n_f2) return;
@@ -397,12 +411,15 @@ struct Ops {
   static void launch_band(const BatchPlan& p, const MemberDev<Real>* m, cudaStream_t s) {
     if (!p.n_band) return;
     if constexpr (!DEV) {
-      if (p.split && p.n_band <= kSplitBlocks) {
-        kb_gamma_split<S><<<4 * p.n_band, 128, 0, s>>>(m, p.band_tab);
+      if (p.fixed) {
+        if (p.split && p.n_band <= kSplitBlocks)
+          kb_gamma_split<S><<<4 * p.n_band, 128, 0, s>>>(m, p.band_tab);
+        else
+          kb_gamma<S, Real, DEV, true><<<p.n_band, 128, 0, s>>>(m, p.band_tab);
         return;
       }
     }
-    kb_gamma<S, Real, DEV><<<p.n_band, 128, 0, s>>>(m, p.band_tab);
+    kb_gamma<S, Real, DEV, false><<<p.n_band, 128, 0, s>>>(m, p.band_tab);
   }
 
   // Boundary-side work forks from d.st: the boundary band on the first stream returned, the PML
@@ -442,8 +459,28 @@ struct Ops {
     constexpr int BY = 4;
     if (nbx <= 0 || ny_in <= 0) return;
     dim3 grid(nbx, (ny_in + BY - 1) / BY);
-    k_bulk<S, Real, DEV, STREAM><<<grid, dim3(32, BY), 0, d.st>>>(
-        g, consts(d), static_cast<const Real*>(d.A), static_cast<Real*>(d.B), d.flag);
+    const Real* A = static_cast<const Real*>(d.A);
+    Real* B = static_cast<Real*>(d.B);
+    if constexpr (!DEV) {
+      if (!STREAM || d.plan->fixed) {
+        k_bulk<S, Real, DEV, STREAM, true><<<grid, dim3(32, BY), 0, d.st>>>(g, consts(d), A, B, d.flag);
+        return;
+      }
+    }
+    k_bulk<S, Real, DEV, STREAM, false><<<grid, dim3(32, BY), 0, d.st>>>(g, consts(d), A, B, d.flag);
+  }
+
+  static void launch_bulk_batch(const BatchPlan& p, const MemberDev<Real>* m, cudaStream_t s) {
+    if (!p.n_bulk) return;
+    const dim3 block(p.tx, p.by);
+    if constexpr (!DEV) {
+      if (p.fixed) {
+        kb_bulk<S, Real, DEV, true>
+            <<<p.n_bulk, block, sizeof(double) * node_smem<S, true>(p.tx * p.by), s>>>(m, p.bulk_tab);
+        return;
+      }
+    }
+    kb_bulk<S, Real, DEV, false><<<p.n_bulk, block, 0, s>>>(m, p.bulk_tab);
   }
 
   // One step of a context: characteristic targets then boundary band, the PML frame, and the
@@ -552,12 +589,12 @@ struct Ops {
   }
 
   static cudaError_t init_eq(const Dev& d, const double* rho, const double* ux, const double* uy,
-                             const double* T) {
+                             const double* T, int* outside) {
     const Geom& g = d.g;
     dim3 grid((g.Lx + 127) / 128, g.Ly);
     k_init_eq<S, Real, DEV><<<grid, 128, 0, d.st>>>(g, consts(d), rho, ux, uy, T,
                                                    static_cast<Real*>(const_cast<void*>(d.A)),
-                                                   static_cast<Real*>(d.Sold));
+                                                   static_cast<Real*>(d.Sold), outside);
     if (g.link && has_pml(g))
       k_init_gamma_s<S, Real, DEV><<<(g.ngamma + 127) / 128, 128, 0, d.st>>>(
           g, consts(d), rho, ux, uy, T, static_cast<Real*>(d.Sold));
@@ -614,8 +651,9 @@ struct Ops {
       }
     }
     if constexpr (!DEV)
-      return cudaFuncSetAttribute(kb_bulk<S, Real, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)sizeof(double) * node_smem<S, Real>(256));
+      return cudaFuncSetAttribute(kb_bulk<S, Real, DEV, true>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(double) * node_smem<S, true>(256));
     if constexpr (DEV) {
       cudaError_t e = cudaFuncSetAttribute(k_pml_fused<S>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
@@ -657,10 +695,11 @@ struct Ops {
     p.by = by;
     p.q = S::Q;
     p.link = n > 0 && dev0[0]->g.link;
-    // the four-warp kernels: FP64 members in fixed point, without PML source terms
+    p.fixed = !DEV && n > 0 && dev0[0]->fixed;
+    // the four-warp kernels: FP64, without PML source terms
     p.split = !DEV;
     for (int m = 0; m < n; ++m)
-      if (!dev0[m]->cd.fx.on || dev0[m]->bc.pml_source & 7) p.split = false;
+      if (dev0[m]->bc.pml_source & 7) p.split = false;
     std::vector<int> bulk, frame, f1, f2, band, tgt, wrap;
     for (int m = 0; m < n; ++m) {
       const Geom& g = dev0[m]->g;
@@ -781,9 +820,7 @@ struct Ops {
     }
     launch_frame2(p, mem, fs);
     // the interiors of every member on st
-    if (p.n_bulk)
-      kb_bulk<S, Real, DEV><<<p.n_bulk, dim3(p.tx, p.by),
-                              sizeof(double) * node_smem<S, Real>(p.tx * p.by), st>>>(mem, p.bulk_tab);
+    launch_bulk_batch(p, mem, st);
     if (aux) {
       cudaEventRecord(join, aux);
       cudaStreamWaitEvent(st, join, 0);
