@@ -129,7 +129,8 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* rho, const double* ux, const dou
                     const double* T, int fields_on_device);
 
 /* Advance n >= 0 time steps (collide with PML, stream, boundary). Asynchronous on the
- * context stream. Returns LBM_EUNSTABLE if an earlier step has already flagged an unphysical
+ * context stream, which must not be under capture (LBM_ECUDA, nothing is launched; the same for
+ * lbm_batch_step). Returns LBM_EUNSTABLE if an earlier step has already flagged an unphysical
  * state (the flag lives in mapped host memory and is read without synchronizing). */
 lbm_status lbm_step(lbm_ctx* ctx, int n);
 

@@ -345,6 +345,14 @@ static void set_form(lbm_ctx* ctx, bool fixed) {
   }
 }
 
+// Steps alternate buffers and are counted on the host, so a caller's graph cannot replay them; the
+// executable graphs that most steps are could not be captured either.
+static bool being_captured(cudaStream_t s) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  return s && cudaStreamIsCapturing(s, &c) == cudaSuccess && c != cudaStreamCaptureStatusNone;
+}
+static const char kCaptured[] = "the stream is being captured: steps cannot be replayed";
+
 static lbm_status check_ready(lbm_ctx* ctx) {
   if (!ctx) return LBM_EINVAL;
   if (!ctx->initialized) { ctx->err = "context not initialized"; return LBM_ESTATE; }
@@ -795,6 +803,7 @@ lbm_status lbm_step(lbm_ctx* ctx, int n) {
   if (s != LBM_OK) return s;
   if (n < 0) { ctx->err = "negative step count"; return LBM_EINVAL; }
   if (*(volatile int*)ctx->hflag) { ctx->err = "unphysical state flagged"; return LBM_EUNSTABLE; }
+  if (n > 0 && being_captured(ctx->st)) { ctx->err = kCaptured; return LBM_ECUDA; }
   for (int k = 0; k < n; ++k) {
     const bool profiled = ctx->prof_used < ctx->prof_cap;
     const bool many = ctx->use_graphs && !profiled && n - k >= kGraphSteps &&
@@ -1322,6 +1331,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int n) {
   if (b->members.empty() || n == 0) return LBM_OK;
   for (lbm_ctx* c : b->members)
     if (*(volatile int*)c->hflag) { b->err = "a member flagged an unphysical state"; return LBM_EUNSTABLE; }
+  if (being_captured(b->st)) { b->err = kCaptured; return LBM_ECUDA; }
   lbm_ctx* ctx = b->members[0];  // for LBM_CK messages
   LBM_CK(cudaSetDevice(b->device));
   for (int k = 0; k < n; ++k) {

@@ -59,3 +59,37 @@ def test_large_fp64_batch_equals_its_members(q, grad):
             s.close()
     for m in range(n):
         assert np.array_equal(got[m], populations(kw, "fp64", states[m], [11]))
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32dev"])
+def test_step_under_capture_is_refused(prec):
+    """Refused without spoiling the caller's capture, and the context goes on as if not called."""
+    import torch
+
+    from paper_2504_20169_gb300 import Solver
+    from paper_2504_20169_gb300._lib import LBMError
+
+    st = torch.cuda.Stream()
+    x = torch.zeros(4, device="cuda")
+    f = wl.random_smooth_state(30, 26, 4, seed=1, du=0.02, mean_u=(0.1, 0.05))
+    args = (30, 26, 4, 0.8, 0.05, 2, "zg", 17, (0, 0, 0, 0), 0.0, (1.0, 0.1, 0.05, 1.0))
+    ref, s = (Solver(*args, precision=prec, stream=st) for _ in range(2))
+    ref.init(*f)
+    ref.step(30)
+    s.init(*f)
+    s.step(13)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        x += 1
+        for n in (1, 17):
+            with pytest.raises(LBMError):
+                s.step(n)
+    g.replay()
+    g.replay()
+    s.step(17)
+    torch.cuda.synchronize()
+    assert torch.all(x == 2)
+    assert np.array_equal(s.export_populations(), ref.export_populations())
+    s.close()
+    ref.close()
