@@ -225,7 +225,7 @@ struct lbm_ctx {
   cudaEvent_t fork = nullptr, join = nullptr, join2 = nullptr, ready = nullptr, begun = nullptr;
   // one step and kGraphSteps steps, keyed by the buffer parity they start from
   cudaGraphExec_t graph[2] = {nullptr, nullptr}, many[2] = {nullptr, nullptr};
-  int singles = 0;
+  int direct = 0;   // steps launched one by one (how)
   bool use_graphs = true;
   std::vector<cudaEvent_t> prof;   // kKernelClasses * 2 events per recorded step
   int prof_cap = 0, prof_used = 0;
@@ -308,12 +308,20 @@ static bool fixed_form(const lbm_ctx* ctx, int outside) {
 // Steps in the longer of a context's (and a batch's) two graphs: even, so that a replay starts and
 // ends with the same buffer parity. Between two graphs of one step the device idles for a fork, a
 // join and a launch, inside one graph for dependent nodes only: a 512^2 FP32 step 66 -> 52 us, a
-// 64^2 FP64 step 32 -> 27 us (2048^2: 287 -> 285). Building it takes 180 us, so the first steps of
-// a context are launched one by one and the device works on them meanwhile.
+// 64^2 FP64 step 32 -> 27 us (2048^2: 287 -> 285). Building it takes 180 us, so the first
+// kDirectSteps steps of a context are launched one by one and the device works on them meanwhile.
 constexpr int kGraphSteps = 8, kDirectSteps = 4;
-// Single steps (calls of fewer than kGraphSteps steps, remainders) launched one by one, about 20 us
-// of host time each, before a context builds the graphs of one step (35 us each, 5 us a launch).
+// Steps launched one by one in all (those first ones, calls of fewer than kGraphSteps steps,
+// remainders), about 20 us of host time each, before a context builds the graphs of one step (35 us
+// each, 5 us a launch).
 constexpr int kSingles = 16;
+
+// How the next of `left` steps is launched after `direct` ones were launched one by one.
+enum class Launch { direct, graph, many };
+static Launch how(int left, int direct, bool have_many, bool have_graph) {
+  if (left >= kGraphSteps && (have_many || direct >= kDirectSteps)) return Launch::many;
+  return have_graph || direct >= kSingles ? Launch::graph : Launch::direct;
+}
 
 static size_t target_slots(const Geom& g) { return 4 * (size_t)g.nb; }
 static size_t edge_slots(const Geom& g) { return 4 * (size_t)g.ne; }
@@ -806,9 +814,11 @@ lbm_status lbm_step(lbm_ctx* ctx, int n) {
   if (n > 0 && being_captured(ctx->st)) { ctx->err = kCaptured; return LBM_ECUDA; }
   for (int k = 0; k < n; ++k) {
     const bool profiled = ctx->prof_used < ctx->prof_cap;
-    const bool many = ctx->use_graphs && !profiled && n - k >= kGraphSteps &&
-                      (ctx->many[ctx->cur] || k >= kDirectSteps);
-    if (many || (ctx->use_graphs && !profiled && ctx->singles >= kSingles)) {
+    const Launch l = !ctx->use_graphs || profiled
+                         ? Launch::direct
+                         : how(n - k, ctx->direct, ctx->many[ctx->cur], ctx->graph[ctx->cur]);
+    if (l != Launch::direct) {
+      const bool many = l == Launch::many;
       cudaGraphExec_t* exec = many ? &ctx->many[ctx->cur] : &ctx->graph[ctx->cur];
       if (!*exec) {
         lbm_status gs = build_graph(ctx, ctx->cur, many ? kGraphSteps : 1, exec);
@@ -821,7 +831,7 @@ lbm_status lbm_step(lbm_ctx* ctx, int n) {
         continue;
       }
     } else {
-      ctx->singles++;
+      ctx->direct++;
       set_roles(ctx, ctx->cur, ctx->scur);
       Dev d = ctx->dev;
       if (profiled) {

@@ -93,3 +93,15 @@ def test_step_under_capture_is_refused(prec):
     assert np.array_equal(s.export_populations(), ref.export_populations())
     s.close()
     ref.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32dev"])
+def test_repeated_short_calls_equal_single_steps(prec):
+    """Calls of 8 to 11 steps: a graph of eight from the second call on, remainders one by one and
+    later by graphs of one."""
+    kw = case_kwargs(nx=33, ny=29, W=4, tau=0.8, sigma_max=0.05, sigma_power=2, bc="nrbc", q=17,
+                     nrbc_edges=(0, 1, 0, 0), beta=0.2, mean=(1.0, 0.1, 0.05, 1.0))
+    f = wl.random_smooth_state(33, 29, 4, seed=2, du=0.02, drho=0.01, dT=0.01, mean_u=(0.1, 0.05))
+    ref = populations(kw, prec, f, [1] * 99)
+    for calls in ([8, 8, 8, 6] * 3 + [9], [9] * 11, [10] * 9 + [9], [11] * 9):
+        assert np.array_equal(populations(kw, prec, f, calls), ref)

@@ -89,3 +89,31 @@ def test_a_stream_being_captured_is_refused(lib, prec):
         assert steps_of(lib, c) == steps_of(lib, other) == done
     lib.lbm_batch_destroy(b)
     lib.lbm_destroy(c), lib.lbm_destroy(other)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_repeated_short_calls_reach_the_graph_of_eight(lib, prec):
+    """Calls of 8 to 11 steps, as a study that samples every ten makes them (after twelve calls the
+    remainders have graphs of their own as well)."""
+    for n in (8, 9, 10, 11):
+        c = context(lib, prec)
+        for _ in range(12):
+            assert lib.lbm_step(c, n) == 0
+        calls(lib)
+        for _ in range(2):                        # n odd: one call from each buffer
+            assert lib.lbm_step(c, n) == 0
+            s = calls(lib)
+            assert s == "G" * (1 + n - 8), (n, s)
+        assert steps_of(lib, c) == 14 * n
+        lib.lbm_destroy(c)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_first_steps_run_while_a_graph_is_built(lib, prec):
+    c = context(lib, prec)
+    calls(lib)
+    assert lib.lbm_step(c, 100) == 0
+    s = calls(lib)
+    per_step = s.index("I") // 4                  # four steps launched one by one, then graphs
+    assert s == "k" * (4 * per_step) + "I" + 12 * "G", s
+    lib.lbm_destroy(c)
