@@ -253,8 +253,8 @@ lbm_status lbm_peak_fma(lbm_precision precision, double* tflops, double* ms, voi
  * lbm_batch_tile sets the interior kernel's block shape tx x by (tx in {32, 64, 128, 256},
  * by >= 1, tx * by <= 256; 0, 0 = the tuned shape for this stencil, precision and device if
  * one was found in this process, else 32 x 4). lbm_batch_autotune times `steps` batch steps
- * with each of the candidate shapes 32x2, 32x4, 32x8, 64x2, 64x4, 128x1, 128x2, 256x1 (one
- * untimed step each to build them), keeps the fastest for this batch, records it for
+ * with each of the candidate shapes 32x2, 32x4, 32x8, 64x2, 64x4, 128x1, 128x2, 256x1 (after one
+ * untimed step each, with the graphs of the timed ones built), keeps the fastest for this batch, records it for
  * (stencil, precision, PML gradient mode, device name) for later batches of the process, and
  * returns it in *tx, *by (either may be NULL). Tuning steps are real steps: every member
  * advances by 8 (steps + 1); the shape never changes the results. */

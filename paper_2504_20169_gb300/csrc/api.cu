@@ -1232,6 +1232,29 @@ static lbm_status batch_graph(lbm_batch* b, int state, int steps, cudaGraphExec_
   return LBM_OK;
 }
 
+// The members' parity state against the plans (0 or 1), or -1: there is no plan for them (a member
+// stepped on its own since then makes the states disagree, one initialized again may have another
+// form).
+static int batch_state(const lbm_batch* b) {
+  if (!b->built) return -1;
+  const int state = b->members[0]->cur != b->base[0] ? 1 : 0;
+  for (size_t m = 0; m < b->members.size(); ++m) {
+    const int s = b->members[m]->cur != b->base[m] ? 1 : 0;
+    if (s != state || b->form[m] != (char)b->members[m]->dev.fixed) return -1;
+  }
+  return state;
+}
+
+// Builds the graphs that the next n steps launch.
+static lbm_status batch_graphs(lbm_batch* b, int n) {
+  int state = batch_state(b);
+  lbm_status s = LBM_OK;
+  if (n >= kGraphSteps && !b->many[state]) s = batch_graph(b, state, kGraphSteps, &b->many[state]);
+  for (int k = 0; k < n % kGraphSteps && s == LBM_OK; ++k, state ^= 1)
+    if (!b->graph[state]) s = batch_graph(b, state, 1, &b->graph[state]);
+  return s;
+}
+
 // Plans for the current member set and tile shape (the graphs follow with the first step).
 static lbm_status batch_build(lbm_batch* b) {
   batch_clear(b);
@@ -1345,17 +1368,8 @@ lbm_status lbm_batch_step(lbm_batch* b, int n) {
   lbm_ctx* ctx = b->members[0];  // for LBM_CK messages
   LBM_CK(cudaSetDevice(b->device));
   for (int k = 0; k < n; ++k) {
-    // parity state of the members against the plans (a member stepped on its own since
-    // then makes the states disagree, one initialized again may have another form: rebuild)
-    int state = -1;
-    if (b->built) {
-      for (size_t m = 0; m < b->members.size(); ++m) {
-        const int s = b->members[m]->cur != b->base[m] ? 1 : 0;
-        if (state < 0) state = s;
-        if (s != state || b->form[m] != (char)b->members[m]->dev.fixed) { state = -2; break; }
-      }
-    }
-    if (!b->built || state < 0) {
+    int state = batch_state(b);
+    if (state < 0) {
       lbm_status bs = batch_build(b);
       if (bs != LBM_OK) return bs;
       state = 0;
@@ -1400,7 +1414,8 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int steps, int* tx_out, int* by_out)
     b->tx = c[0];
     b->by = c[1];
     batch_clear(b);
-    st = lbm_batch_step(b, 1);   // builds the plan and graphs (one untimed step)
+    st = lbm_batch_step(b, 1);   // builds the plan (one untimed step)
+    if (st == LBM_OK) st = batch_graphs(b, steps);
     if (st != LBM_OK) break;
     cudaEventRecord(e0, b->st);
     st = lbm_batch_step(b, steps);

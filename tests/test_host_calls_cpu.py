@@ -117,3 +117,17 @@ def test_first_steps_run_while_a_graph_is_built(lib, prec):
     per_step = s.index("I") // 4                  # four steps launched one by one, then graphs
     assert s == "k" * (4 * per_step) + "I" + 12 * "G", s
     lib.lbm_destroy(c)
+
+
+@pytest.mark.parametrize("steps", [1, 2, 5, 8, 11])
+def test_autotune_times_steps_alone(lib, steps):
+    """Nothing is built between the two events around a candidate's timed steps."""
+    c = context(lib, 1)
+    b = batch(lib, [c])
+    calls(lib)
+    assert lib.lbm_batch_autotune(b, steps, None, None) == 0
+    regions = re.findall(r"R([^RT]*)RT", calls(lib))
+    assert regions == ["G" * (steps // 8 + steps % 8)] * 8, regions
+    assert steps_of(lib, c) == 8 * (steps + 1)
+    lib.lbm_batch_destroy(b)
+    lib.lbm_destroy(c)
