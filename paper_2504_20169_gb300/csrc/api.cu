@@ -309,7 +309,8 @@ static bool fixed_form(const lbm_ctx* ctx, int outside) {
 // ends with the same buffer parity. Between two graphs of one step the device idles for a fork, a
 // join and a launch, inside one graph for dependent nodes only: a 512^2 FP32 step 66 -> 52 us, a
 // 64^2 FP64 step 32 -> 27 us (2048^2: 287 -> 285). Building it takes 180 us, so the first
-// kDirectSteps steps of a context are launched one by one and the device works on them meanwhile.
+// kDirectSteps steps of a context, and of a batch after a change of members, are launched one by one
+// and the device works on them meanwhile.
 constexpr int kGraphSteps = 8, kDirectSteps = 4;
 // Steps launched one by one in all (those first ones, calls of fewer than kGraphSteps steps,
 // remainders), about 20 us of host time each, before a context builds the graphs of one step (35 us
@@ -1184,6 +1185,7 @@ struct lbm_batch {
   std::vector<char> form;                 // when the plans were built
   std::vector<BatchGroup> groups;
   cudaGraphExec_t graph[2] = {nullptr, nullptr}, many[2] = {nullptr, nullptr};
+  int direct = 0;                         // steps launched one by one since then (how)
   int tx = 0, by = 0;                     // bulk tile shape; 0: from the tuning cache / default
   bool built = false;
   std::string err;
@@ -1196,6 +1198,7 @@ static void batch_clear(lbm_batch* b) {
   }
   for (auto& g : b->groups) batch_plan_free(&g.plan);
   b->groups.clear();
+  b->direct = 0;
   b->built = false;
 }
 
@@ -1208,15 +1211,21 @@ static std::tuple<int, int, int, std::string> tune_key(const lbm_ctx* c) {
   return {c->q, (int)c->prec, c->g.link, device_name(c->device)};
 }
 
+// Launches one step of every group from a parity state on s.
+static cudaError_t batch_launch(lbm_batch* b, int state, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  for (auto& G : b->groups)
+    if (e == cudaSuccess)
+      e = G.ops.batch_step(G.plan, state, s, b->aux, b->aux2, b->fork, b->join, b->join2, b->begun);
+  return e;
+}
+
 // `steps` steps of every group from a parity state on, as an executable graph.
 static lbm_status batch_graph(lbm_batch* b, int state, int steps, cudaGraphExec_t* exec) {
   cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
-    for (int k = 0; k < steps; ++k)
-      for (auto& G : b->groups)
-        if (e == cudaSuccess)
-          e = G.ops.batch_step(G.plan, (state + k) & 1, b->cap, b->aux, b->aux2, b->fork, b->join,
-                               b->join2, b->begun);
+    for (int k = 0; k < steps && e == cudaSuccess; ++k)
+      e = batch_launch(b, (state + k) & 1, b->cap);
     cudaGraph_t graph = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);
     if (e == cudaSuccess) e = e2;
@@ -1374,13 +1383,19 @@ lbm_status lbm_batch_step(lbm_batch* b, int n) {
       if (bs != LBM_OK) return bs;
       state = 0;
     }
-    const bool many = n - k >= kGraphSteps;
-    cudaGraphExec_t* exec = many ? &b->many[state] : &b->graph[state];
-    if (!*exec) {
-      lbm_status gs = batch_graph(b, state, many ? kGraphSteps : 1, exec);
-      if (gs != LBM_OK) return gs;
+    const Launch l = how(n - k, b->direct, b->many[state], b->graph[state]);
+    const bool many = l == Launch::many;
+    if (l == Launch::direct) {
+      LBM_CK(batch_launch(b, state, b->st));
+      b->direct++;
+    } else {
+      cudaGraphExec_t* exec = many ? &b->many[state] : &b->graph[state];
+      if (!*exec) {
+        lbm_status gs = batch_graph(b, state, many ? kGraphSteps : 1, exec);
+        if (gs != LBM_OK) return gs;
+      }
+      LBM_CK(cudaGraphLaunch(*exec, b->st));
     }
-    LBM_CK(cudaGraphLaunch(*exec, b->st));
     const int done = many ? kGraphSteps : 1;
     for (lbm_ctx* c : b->members) {
       if (!many) {

@@ -131,3 +131,25 @@ def test_autotune_times_steps_alone(lib, steps):
     assert steps_of(lib, c) == 8 * (steps + 1)
     lib.lbm_batch_destroy(b)
     lib.lbm_destroy(c)
+
+
+def test_a_batch_builds_its_graph_behind_running_steps(lib):
+    """After a change of members the first steps are launched one by one, and a chunk of a hundred
+    steps builds one graph."""
+    c, d = context(lib, 1), context(lib, 1)
+    b = batch(lib, [c])
+    for members in ([c], [c, d]):
+        assert lib.lbm_batch_set(b, (C.c_void_p * len(members))(*[m.value for m in members]),
+                                 len(members)) == 0
+        calls(lib)
+        assert lib.lbm_batch_step(b, 100) == 0
+        s = calls(lib)
+        per_step = s.index("I") // 4
+        assert per_step > 0 and s == "k" * (4 * per_step) + "I" + "G" * 12, s
+        assert lib.lbm_batch_step(b, 1) == 0
+        assert calls(lib) == "k" * per_step
+        assert lib.lbm_batch_step(b, 9) == 0      # from the other buffer
+        assert calls(lib) == "IG" + "k" * per_step
+    assert (steps_of(lib, c), steps_of(lib, d)) == (220, 110)
+    lib.lbm_batch_destroy(b)
+    lib.lbm_destroy(c), lib.lbm_destroy(d)
