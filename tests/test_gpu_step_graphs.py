@@ -105,3 +105,32 @@ def test_repeated_short_calls_equal_single_steps(prec):
     ref = populations(kw, prec, f, [1] * 99)
     for calls in ([8, 8, 8, 6] * 3 + [9], [9] * 11, [10] * 9 + [9], [11] * 9):
         assert np.array_equal(populations(kw, prec, f, calls), ref)
+
+
+@pytest.mark.parametrize("q,grad,n", [(37, "central", 26), (17, "link", 26), (9, "central", 70)])
+def test_larger_fp64_batch_equals_its_members(q, grad, n):
+    """The band too in more blocks than the split kernel takes (above 256; a member has 11, on D2Q9
+    4)."""
+    import torch
+
+    from paper_2504_20169_gb300.serving import Batch
+
+    kw = case_kwargs(nx=96, ny=80, W=8, tau=0.8, sigma_max=0.05, sigma_power=2, bc="nrbc", q=q,
+                     pml_grad=grad, nrbc_edges=(0, 1, 0, 1), beta=0.2, mean=(1.0, 0.1, 0.0, 1.0))
+    states = [wl.random_smooth_state(96, 80, 8, seed=m, du=0.02, drho=0.01, dT=0.01,
+                                     mean_u=(0.1, 0.0)) for m in range(3)]
+    alone = [populations(kw, "fp64", f, [11]) for f in states]
+    solvers = [make_solver(kw, "fp64") for _ in range(n)]
+    try:
+        for m, s in enumerate(solvers):
+            s.init(*states[m % 3])
+        batch = Batch()
+        batch.set(solvers)
+        batch.step(11)
+        torch.cuda.synchronize()
+        batch.close()
+        for m, s in enumerate(solvers):
+            assert np.array_equal(s.export_populations(), alone[m % 3]), m
+    finally:
+        for s in solvers:
+            s.close()
