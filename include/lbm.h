@@ -222,7 +222,7 @@ lbm_status lbm_estimate_bytes_bc(const lbm_grid* grid, lbm_stencil stencil, int 
  * [i][y][x]. lbm_export_site_class: per node of F (host buffers of Lx * Ly, layout [y][x], any
  * may be NULL): layer = the PML layer index max(i_x, i_y) (0 in the bulk), has_q = 1 where the
  * PML accumulator Q is kept (P and its inner ring), sigma_x / sigma_y = the absorption
- * coefficients the collision applies (0 off P). Both allocate a temporary device buffer and
+ * coefficients the collision applies (0 off P), in the context's precision. Both allocate a temporary device buffer and
  * synchronize the context stream. */
 lbm_status lbm_export_pull_index(lbm_ctx* ctx, int64_t* host);
 lbm_status lbm_export_site_class(lbm_ctx* ctx, int32_t* layer, uint8_t* has_q, double* sigma_x,

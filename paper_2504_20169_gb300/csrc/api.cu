@@ -967,19 +967,19 @@ __global__ void k_pull_index(Geom g, long long* __restrict__ out) {
   }
 }
 
-__global__ void k_site_class(Geom g, Consts<double> c, int* __restrict__ layer,
+template <class Real>
+__global__ void k_site_class(Geom g, Consts<Real> c, int* __restrict__ layer,
                              unsigned char* __restrict__ hasq, double* __restrict__ sxo,
                              double* __restrict__ syo) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   if (x >= g.Lx) return;
-  const PmlNode<double> n = pml_node<double>(g, x, y);
+  const PmlNode<Real> n = pml_node<Real>(g, x, y);
+  const PmlLayers<Real> p = pml_layers(g, c, x, y);
   const long long k = (long long)y * g.Lx + x;
   layer[k] = max(n.ix, n.iy);
-  hasq[k] = has_pml(g) && n.has_q ? 1 : 0;
-  double sx = 0.0, sy = 0.0;
-  if (n.in_p) pml_sigmas(c, n, sx, sy);
-  sxo[k] = sx;
-  syo[k] = sy;
+  hasq[k] = has_pml(g) && p.has_q ? 1 : 0;
+  sxo[k] = p.in_p ? double(p.sx) : 0.0;
+  syo[k] = p.in_p ? double(p.sy) : 0.0;
 }
 }  // namespace lbm
 
@@ -1017,7 +1017,11 @@ lbm_status lbm_export_site_class(lbm_ctx* ctx, int32_t* layer, uint8_t* has_q, d
   double* sy = sx + n;
   int* ly = reinterpret_cast<int*>(sy + n);
   unsigned char* hq = reinterpret_cast<unsigned char*>(ly + n);
-  k_site_class<<<dim3((g.Lx + 127) / 128, g.Ly), 128, 0, ctx->st>>>(g, ctx->dev.cd, ly, hq, sx, sy);
+  const dim3 grid((g.Lx + 127) / 128, g.Ly);
+  if (ctx->prec == LBM_FP64)
+    k_site_class<double><<<grid, 128, 0, ctx->st>>>(g, ctx->dev.cd, ly, hq, sx, sy);
+  else
+    k_site_class<float><<<grid, 128, 0, ctx->st>>>(g, ctx->dev.cf, ly, hq, sx, sy);
   cudaError_t e = cudaGetLastError();
   auto get = [&](void* dst, const void* src, size_t b) {
     if (dst && e == cudaSuccess) e = cudaMemcpyAsync(dst, src, b, cudaMemcpyDeviceToHost, ctx->st);

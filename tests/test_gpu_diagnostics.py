@@ -68,3 +68,25 @@ def test_fma_peaks_are_measured():
     print(f"FMA peak: FP64 {f64:.3f} TFLOP/s ({ms64:.1f} ms), FP32 {f32:.2f} TFLOP/s ({ms32:.1f} ms)")
     assert 0.1 < f64 < 100.0 and 10.0 < f32 < 200.0
     assert f32 > 5 * f64
+
+
+@pytest.mark.parametrize("widths,py,split,grad", [((5, 5, 5, 5), False, False, "central"),
+                                                  ((4, 7, 0, 3), False, True, "central"),
+                                                  ((6, 3, 2, 5), False, False, "link"),
+                                                  ((3, 6, 0, 0), True, False, "central")])
+def test_site_class_is_what_fp32_kernels_read(widths, py, split, grad):
+    """The sigma of an FP32 context is that of its table: single precision, formed as (i / W)^p."""
+    nx, ny, smax, p = 21, 18, 0.3, 3
+    kw = case_kwargs(nx=nx, ny=ny, W=widths[0], widths=widths, sigma_max=smax, sigma_power=p,
+                     periodic_y=py, split=split, pml_grad=grad)
+    with make_solver(kw, "fp32dev") as s:
+        layer, hq, sx, sy = s.site_class()
+    with make_solver(kw, "fp64") as s:
+        layer64, hq64, sx64, sy64 = s.site_class()
+    assert np.array_equal(layer, layer64) and np.array_equal(hq, hq64)
+    for a, b in ((sx, sx64), (sy, sy64)):
+        assert np.array_equal(a, a.astype(np.float32)) and np.allclose(a, b, rtol=1e-6, atol=0)
+    f = np.float32
+    for i in range(1, widths[0] + 1):               # the W edge's layers at mid height
+        want = f(smax) * (f(i) / f(widths[0])) ** 3
+        assert abs(sx[ny // 2 + widths[2], widths[0] - i] - want) <= 2e-7 * want
