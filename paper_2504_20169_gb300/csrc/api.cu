@@ -582,7 +582,9 @@ lbm_status lbm_create(const lbm_grid* grid, lbm_stencil stencil, double tau, int
   if (dalloc(ctx, (void**)&ctx->partials, sizeof(double) * 12 * (size_t)ctx->max_blocks) !=
       cudaSuccess)
     return oom("partials");
-  if (dalloc(ctx, (void**)&ctx->dout, sizeof(double) * 16) != cudaSuccess) return oom("outputs");
+  if (dalloc(ctx, (void**)&ctx->dout, sizeof(double) * 16) != cudaSuccess ||
+      cudaMemsetAsync(ctx->dout, 0, sizeof(double) * 16, ctx->st) != cudaSuccess)
+    return oom("outputs");
   if (cudaHostAlloc(&ctx->hout, sizeof(double) * 16, cudaHostAllocDefault) != cudaSuccess)
     return oom("pinned outputs");
   if (cudaHostAlloc(&ctx->hflag, sizeof(int), cudaHostAllocMapped) != cudaSuccess)
@@ -762,10 +764,13 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* rho, const double* ux, const dou
   *ctx->hflag = 0;
   Dev& d = ctx->dev;
   set_roles(ctx, 0, 0);
-  int* outside = reinterpret_cast<int*>(ctx->dout + 15);   // past the reductions' twelve values
-  LBM_CK(cudaMemsetAsync(outside, 0, sizeof(int), ctx->st));
+  // FP64: a count past the reductions' twelve values, zero between calls
+  const bool fp64 = ctx->prec == LBM_FP64;
+  int* outside = reinterpret_cast<int*>(ctx->dout + 15);
+  int* n_outside = reinterpret_cast<int*>(ctx->hout + 15);
+  *n_outside = 0;
   LBM_CK(ctx->ops.init_eq(d, src[0], src[1], src[2], src[3], outside));
-  LBM_CK(cudaMemcpyAsync(ctx->hout + 15, outside, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+  if (fp64) LBM_CK(cudaMemcpyAsync(n_outside, outside, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
   if (ctx->bc == LBM_BC_NRBC) {
     k_init_targets<<<(g.nb + 127) / 128, 128, 0, ctx->st>>>(g, src[0], src[1], src[2], src[3],
                                                             d.Vtgt);
@@ -774,7 +779,8 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* rho, const double* ux, const dou
   // initial collision (no streaming): buffer 0 holds f^0, buffer 1 receives f*^0
   LBM_CK(ctx->ops.step(d, false));
   LBM_CK(cudaStreamSynchronize(ctx->st));
-  set_form(ctx, fixed_form(ctx, *reinterpret_cast<const int*>(ctx->hout + 15)));
+  if (*n_outside) LBM_CK(cudaMemsetAsync(outside, 0, sizeof(int), ctx->st));
+  set_form(ctx, fixed_form(ctx, *n_outside));
   ctx->cur = 1;
   ctx->scur = 1;
   ctx->steps = 0;
@@ -1185,8 +1191,8 @@ struct lbm_batch {
   cudaEvent_t fork = nullptr, join = nullptr, join2 = nullptr, begun = nullptr;
   int device = -1;
   std::vector<lbm_ctx*> members;
-  std::vector<int> base;                  // members' buffer parity and FP64 form (Dev::fixed)
-  std::vector<char> form;                 // when the plans were built
+  std::vector<int> base;                  // members' buffer parity when the plans were built
+  std::vector<char> form;                 // and their FP64 form (Dev::fixed)
   std::vector<BatchGroup> groups;
   cudaGraphExec_t graph[2] = {nullptr, nullptr}, many[2] = {nullptr, nullptr};
   int direct = 0;                         // steps launched one by one since then (how)
