@@ -194,8 +194,9 @@ lbm_status lbm_restore(lbm_ctx* ctx, const void* host, size_t bytes);
  * targets, 1 interior (BGK only), 2 PML frame phase 1, 3 PML frame phase 2, 4 boundary band;
  * max_steps = 0 disables. Recorded steps are launched directly with every class running alone
  * (no concurrency between the interior kernel and the boundary chain), so each class's time
- * is its own; unrecorded steps keep the concurrent graph replay. lbm_profile_read synchronizes, writes the summed GPU milliseconds of
- * each class into ms[5] and the number of recorded steps into *steps, and restarts recording. */
+ * is its own; unrecorded steps run concurrently as ever. lbm_profile_read synchronizes, writes the
+ * summed GPU milliseconds of each class into ms[5] and the number of recorded steps into *steps, and
+ * restarts recording. */
 lbm_status lbm_profile_enable(lbm_ctx* ctx, int max_steps);
 lbm_status lbm_profile_read(lbm_ctx* ctx, double* ms, int* steps);
 
@@ -222,14 +223,14 @@ lbm_status lbm_estimate_bytes_bc(const lbm_grid* grid, lbm_stencil stencil, int 
  * [i][y][x]. lbm_export_site_class: per node of F (host buffers of Lx * Ly, layout [y][x], any
  * may be NULL): layer = the PML layer index max(i_x, i_y) (0 in the bulk), has_q = 1 where the
  * PML accumulator Q is kept (P and its inner ring), sigma_x / sigma_y = the absorption
- * coefficients the collision applies (0 off P), in the context's precision. Both allocate a temporary device buffer and
- * synchronize the context stream. */
+ * coefficients the collision applies (0 off P), in the context's precision. Both allocate a
+ * temporary device buffer and synchronize the context stream. */
 lbm_status lbm_export_pull_index(lbm_ctx* ctx, int64_t* host);
 lbm_status lbm_export_site_class(lbm_ctx* ctx, int32_t* layer, uint8_t* has_q, double* sigma_x,
                                  double* sigma_y);
 
-/* Measured vector FMA throughput of the current CUDA device (no counterpart in the paper: the
- * ALU roofline of the FP64 path, whose interior kernel is bound by the FP64 pipe). precision
+/* Measured vector FMA throughput of the current CUDA device (no counterpart in the paper; what the
+ * rate of the FP64 path, which updates its nodes in fixed point, is put beside). precision
  * LBM_FP64 times double FMAs, LBM_FP32_DEV float FMAs: every SM filled with threads running
  * eight independent FMA chains, one warm-up launch, then one timed launch (CUDA events on
  * cuda_stream, a cudaStream_t or NULL). *tflops = 2 x FMAs / time, *ms = the timed launch
@@ -238,13 +239,14 @@ lbm_status lbm_peak_fma(lbm_precision precision, double* tflops, double* ms, voi
 
 /* Batched execution of independent instances (serving). A batch holds a resident set of
  * initialized contexts on one device and advances all of them together. Members are grouped
- * by (stencil, precision, PML gradient mode); within a group every kernel class (characteristic
- * targets, interior, PML frame, boundary band, periodic row copies) is one launch whose blocks
- * walk a table of (member, tile) entries spanning all members of the group, so instances of
+ * by (stencil, precision, PML gradient mode, FP64 form); within a group every kernel class
+ * (characteristic targets, interior, PML frame, boundary band, periodic row copies) is one launch
+ * whose blocks walk a table of (member, tile) entries spanning all members of the group, so instances of
  * different sizes, PML widths and boundary conditions share each launch and fill the GPU
- * together; one step of the whole batch is one CUDA-graph launch on the batch's stream. Each
- * block runs the same per-node code as lbm_step, so every member computes bit for bit what it
- * computes alone, whatever the tile shape. lbm_batch_set replaces the resident set (continuous
+ * together; eight steps of the whole batch are one CUDA-graph launch on the batch's stream, the
+ * first steps after a change of members and remainders of a call single ones. Each block runs the
+ * same per-node code as lbm_step, so every member computes bit for bit what it computes alone,
+ * whatever the tile shape. lbm_batch_set replaces the resident set (continuous
  * batching: call it between steps as instances are admitted or retired; the plans and graphs are
  * rebuilt on the next step, as they are when a member was stepped on its own in between).
  * lbm_batch_step returns LBM_EUNSTABLE without stepping anyone if a member has flagged an
@@ -254,8 +256,8 @@ lbm_status lbm_peak_fma(lbm_precision precision, double* tflops, double* ms, voi
  * by >= 1, tx * by <= 256; 0, 0 = the tuned shape for this stencil, precision and device if
  * one was found in this process, else 32 x 4). lbm_batch_autotune times `steps` batch steps
  * with each of the candidate shapes 32x2, 32x4, 32x8, 64x2, 64x4, 128x1, 128x2, 256x1 (after one
- * untimed step each, with the graphs of the timed ones built), keeps the fastest for this batch, records it for
- * (stencil, precision, PML gradient mode, device name) for later batches of the process, and
+ * untimed step each, with the graphs of the timed ones built), keeps the fastest for this batch,
+ * records it for (stencil, precision, PML gradient mode, device name) for later batches of the process, and
  * returns it in *tx, *by (either may be NULL). Tuning steps are real steps: every member
  * advances by 8 (steps + 1); the shape never changes the results. */
 typedef struct lbm_batch lbm_batch;

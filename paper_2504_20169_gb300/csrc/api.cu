@@ -161,10 +161,13 @@ void mean_equilibrium(const double* w, double r, const lbm_bc_params& bp, double
 
 int halo_of(int q) { return q == 9 ? 1 : 3; }
 
-// Fixed-point constants of an FP64 context (fixed.cuh), from the doubles that the FP64 arithmetic
-// multiplies by: the sums of these miss the quadrature by 1e-16, so T drifts by 3e-16 a step, and
-// both arithmetics then drift alike. They stay off where that arithmetic does
-// not apply: omega outside (0, 2), a mean density beyond 2^60 or a mean equilibrium beyond 2^59 units.
+// Fixed-point constants of an FP64 context (fixed.cuh), from the doubles that lbm_lattice_info
+// returns and the FP64 arithmetic multiplies by. Their sums miss the quadrature by up to 2e-16, so
+// energy drifts by that in every step: the scheme with these constants does, and the fixed-point
+// form follows it closely (100 steps of nearly uniform flows, rms against a 64-bit run of the scheme:
+// 5e-16 to 2e-15; FP64 arithmetic, whose own roundings add to it or hold it still, 3e-15 to 1.3e-14).
+// They stay off where that arithmetic does not apply: omega outside (0, 2), a mean density beyond
+// 2^60 or a mean equilibrium beyond 2^59 units.
 template <class S>
 void fixed_consts(const double* w, double r2, double omega, const lbm_bc_params& bp,
                   const double* fbar, fx::Consts& c) {
@@ -770,7 +773,8 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* rho, const double* ux, const dou
   int* n_outside = reinterpret_cast<int*>(ctx->hout + 15);
   *n_outside = 0;
   LBM_CK(ctx->ops.init_eq(d, src[0], src[1], src[2], src[3], outside));
-  if (fp64) LBM_CK(cudaMemcpyAsync(n_outside, outside, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+  if (fp64)
+    LBM_CK(cudaMemcpyAsync(n_outside, outside, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
   if (ctx->bc == LBM_BC_NRBC) {
     k_init_targets<<<(g.nb + 127) / 128, 128, 0, ctx->st>>>(g, src[0], src[1], src[2], src[3],
                                                             d.Vtgt);
@@ -1097,11 +1101,12 @@ lbm_status lbm_checkpoint(lbm_ctx* ctx, void* host, size_t bytes) {
   lbm_checkpoint_size(ctx, &need);
   if (!host || bytes < need) { ctx->err = "checkpoint buffer too small"; return LBM_EINVAL; }
   char* p = static_cast<char*>(host);
+  const bool own_form = ctx->dev.fixed == (ctx->prec == LBM_FP64 && ctx->dev.cd.fx.on);
   CkptHeader h{kMagic, ctx->q, ctx->g.nx, ctx->g.ny, pack_widths(ctx), (int64_t)ctx->prec,
                ctx->steps,
                (int64_t)(ctx->prev_valid ? 1 : 0) | (int64_t)(ctx->prev_prestream ? 2 : 0) |
                    ((int64_t)ctx->g.py << 2) | ((int64_t)ctx->g.link << 3) |
-                   (int64_t)(ctx->dev.fixed != (ctx->prec == LBM_FP64 && ctx->dev.cd.fx.on) ? 16 : 0)};
+                   (int64_t)(own_form ? 0 : 16)};   // 16: all nodes in FP64 (BatchPlan::fixed)
   std::memcpy(p, &h, sizeof h);
   p += sizeof h;
   const cudaMemcpyKind k = cudaMemcpyDeviceToHost;

@@ -551,8 +551,8 @@ __device__ __forceinline__ void bulk_node(const Geom& g, const Consts<Real>& c,
   }
 }
 
-// Blocks of 128 threads per SM of the fixed-point interior. The update is bound by integer issue (about
-// 4500 instructions per D2Q37 node), so more warps help little. Measured at 1024^2, blocks per SM:
+// Blocks of 128 threads per SM of the fixed-point interior. The update is bound by integer issue
+// (about 4500 instructions per D2Q37 node), so more warps help little. Measured at 1024^2, blocks per SM:
 // D2Q37 3 236 us (before the out-of-line FP64 form), 4 202, 5 199 (all its shared memory allows);
 // D2Q17 5 120, 6 95, 8 95, 10 97; D2Q9 8 53, 10 54. In FP64 arithmetic 738, 385 and 203 us.
 template <class S, bool FIXED>
@@ -855,7 +855,7 @@ __device__ __forceinline__ void frame1_split(const Geom& g, const Consts<double>
   }
 }
 
-// Blocks of 128 threads per SM of the fixed-point frame and band kernels. Measured on the 1024^2 frame,
+// Blocks of 128 threads per SM of the fixed-point frame and band kernels. On the 1024^2 frame,
 // phase 1: D2Q37 3 116 us, 4 107, 5 (spills) 124; in FP64 arithmetic 275 us.
 template <class S, bool FIXED>
 constexpr int edge_blocks() {
@@ -894,7 +894,7 @@ __device__ __forceinline__ void frame2_node(const Geom& g, const Consts<Real>& c
   // STAGE: the FP32 kernel, which only the link gradient launches (the printed one has its frame in
   // one kernel). Without the printed form beside it the compiler keeps the addresses of the stores
   // (124 registers instead of 106, still four blocks an SM): the batched sweep of 16 members
-  // 1056 -> 1005 us a step.
+  // 1056 -> 1005 us a step, all else as here (1026 before this kernel took both forms in one).
   if (STAGE || g.link) {
     // link mode: the remaining -sigma Q_i(x + e_i) of -sigma (Q_i(x + e_i) - Q_i(x)), the
     // integral of sigma c_i . grad Q_i along the link the population travels (sigma_x =

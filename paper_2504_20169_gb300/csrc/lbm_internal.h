@@ -16,7 +16,7 @@ struct Dev {
   Consts<float> cf;
   const void* A;     // post-collision populations of the current level (read)
   void* B;           // next level (written)
-  void* Sold;        // PML accumulator S^(n-1) (link mode: Q^n in place during the step)
+  void* Sold;        // PML accumulator S^(n-1) (two-pass frames: Q^n in place during the step)
   void* Snew;        // S^n
   // characteristic targets U_tgt [4][nb], two buffers: a chunk of an edge band also reads its
   // neighbours' targets of level n (Vtgt_in), so those of level n + 1 go to the other one (Vtgt)

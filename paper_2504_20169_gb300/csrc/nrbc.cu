@@ -75,7 +75,8 @@ __device__ inline void char_rate(const BcParams& bc, int variant, double out, co
 // bands wrap around (central tangential differences everywhere, halo taken modulo Ly).
 constexpr int kChunk = 32, kHalo = 4, kText = kChunk + 2 * kHalo;
 
-// (nrbc_chunk is the per-block work; chunk = index over the four bands' chunks, sm = 16 M kText doubles of shared memory.)
+// (nrbc_chunk is the per-block work; chunk = index over the four bands' chunks, sm = 16 M kText
+// doubles of shared memory.)
 template <class R>
 __device__ __forceinline__ void nrbc_chunk(const Geom& g, const BcParams& bc,
                                            const double* __restrict__ Ue,

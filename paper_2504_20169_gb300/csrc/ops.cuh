@@ -367,13 +367,22 @@ __global__ void __launch_bounds__(256) kb_wrap_y(const MemberDev<Real>* __restri
 // it is full. Measured, FP64, one warp / four warps on a node: 64^2 grid (20 blocks) phase 1 33 / 15
 // us, phase 2 26 / 14, band 20 / 13; 300^2 D2Q17 (209 blocks) 22.7 / 20.1, 20.2 / 18.3, 14.2 / 12.1;
 // 1024^2 (band 103 blocks) 32 / 23, (phase 1 1088 blocks) 109 / 139. The interior gains nothing at
-// any size (128^2: 12.5 / 12.6 us).
+// any size (128^2: 12.5 / 12.6 us). The line is one for all lattices and boundaries and too coarse
+// for some: within it the frame's kernels gain on D2Q37 (us a step, one warp / four: 64 + 2 x 8 nodes
+// a side 55 / 24, 300 + 2 x 20 95 / 87; at 253 blocks 95 / 99), on the others without characteristic
+// targets up to 170 blocks (D2Q17 28 / 16, 40 / 39 at 210, 41 / 46 at 253; D2Q9 19 / 12, 24 / 21 at
+// 170, 25 / 29 at 253), and with CBC relax there, where the targets are the critical path, hardly at
+// all (D2Q17 29 / 29 at 20 blocks, 32 / 38 at 115, 39 / 45 at 210). The band gains where it is waited
+// for (link gradient, or targets on small grids) and loses up to a tenth with zero gradient or from
+// some 30 blocks on (D2Q37 800^2: 246 / 281).
 constexpr int kSplitBlocks = 256;
 
 // Tiles of the fused FP32 frame up to which the interior waits for the frame's last block to start
-// (launch_begun): twelve waves of two blocks to each of 152 SMs. Beyond, that wait costs more than
-// the order gives (us a step, waiting / not: 2430 tiles, 4096^2 + PML 32, 895 / 900; 3640, 3072^2 +
-// 64, 645 / 643; 4830, 4096^2 + 64, 1044 / 1032; 9570, 8192^2 + 64, 3571 / 3501). A batch, whose
+// (launch_begun): on D2Q37 twelve waves of two blocks to each of 152 SMs. Beyond, that wait costs
+// more than the order gives (D2Q37, us a step, waiting / not: 2430 tiles, 4096^2 + PML 32, 895 / 900;
+// 3640, 3072^2 + 64, 645 / 643; 4830, 4096^2 + 64, 1044 / 1032; 9570, 8192^2 + 64, 3571 / 3501). The
+// other lattices have more blocks on an SM and could wait for longer: 4096^2 + 64 D2Q17 487 / 485,
+// D2Q9 269 / 276; 8192^2 + 64 1601 / 1601, 879 / 878. A batch, whose
 // interiors are small beside its frames, always waits (16 members, 5000 tiles, 847 / 858).
 constexpr int kFrameFirst = 12 * 304;
 

@@ -3,8 +3,8 @@
 Requests (independent solves of different grid sizes, PML widths and boundary conditions)
 arrive over time. The loop admits queued requests whenever their estimated device footprint
 (lbm_estimate_bytes) fits in the HBM budget, keeps their populations resident, and advances
-every resident instance together through an lbm_batch (one combined CUDA-graph launch per
-step). Admission and retirement happen between chunks of steps, so requests that arrive while
+every resident instance together through an lbm_batch (combined launches, in CUDA graphs of
+eight steps). Admission and retirement happen between chunks of steps, so requests that arrive while
 others are on the GPU join the running batch as memory frees up. An instance that flags an
 unphysical state is retired with status "unstable" without affecting the others.
 """
